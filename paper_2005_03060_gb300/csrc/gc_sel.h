@@ -17,13 +17,18 @@ struct gc_sel {
     std::vector<int32_t> pair_i, pair_j, pair_type;   // [P]
     std::vector<int32_t> win_t0, win_t1;              // [n_ubl]
     // neighbour table [2][n_ubl][N]: pair index with antenna i as i_p (0) or
-    // as j_p (1), -1 if none; empty when it would exceed 16 M entries
+    // as j_p (1), -1 if none; empty when it would exceed 16 M entries, and for
+    // full grids of more than 64 types
     std::vector<int32_t> nbr;
     // X-engine work groups (types sharing a window, <= GC_XENG_NTY each)
     int n_groups = 0, n_windows = 0;
     std::vector<int32_t> grp_types;  // type indices, grouped
     std::vector<int32_t> grp_off;    // [n_groups + 1]
     std::vector<int32_t> grp_t0, grp_t1, grp_first, grp_win, grp_dymax;   // [n_groups]
+    // window entries of the pair-list X-engine (selections with several
+    // windows; empty otherwise): per window its pairs (order_entries), then
+    // P + j for every antenna j
+    std::vector<int32_t> wp_entry, wp_off, wp_t0, wp_t1;
     // arrays on a partly occupied lattice (gc_selection_subset_masked)
     int lattice = 0;                 // 0 square, 1 triangular
     int masked = 0;                  // 1: only the points of `mask` hold antennas
@@ -40,7 +45,8 @@ struct gc_sel {
             *d_pair_type = nullptr, *d_win_t0 = nullptr, *d_win_t1 = nullptr, *d_grp_types = nullptr,
             *d_grp_off = nullptr, *d_grp_t0 = nullptr, *d_grp_t1 = nullptr, *d_grp_first = nullptr,
             *d_grp_win = nullptr, *d_nbr = nullptr, *d_grp_dymax = nullptr, *d_mask = nullptr,
-            *d_tree_ant = nullptr, *d_tree_pair = nullptr, *d_tree_sign = nullptr;
+            *d_tree_ant = nullptr, *d_tree_pair = nullptr, *d_tree_sign = nullptr, *d_wp_entry = nullptr,
+            *d_wp_off = nullptr, *d_wp_t0 = nullptr, *d_wp_t1 = nullptr;
 };
 
 gc_status gc_sel_upload(gc_ctx *ctx, gc_sel *s);
@@ -51,3 +57,18 @@ bool gc_xeng_tc_eligible(const gc_sel *sel, int vfmt, const void *volt, int L);
 int gc_xeng_tc_slices(const gc_ctx *ctx, const gc_sel *sel, int L, int C);
 gc_status gc_xeng_tc_launch(gc_ctx *ctx, const void *volt, int L, int C, int T, const gc_sel *sel, void *part,
                             void *apart, int n_tsplit, cudaStream_t s);
+
+// X-engine over pair lists (gc_xeng_pairs.cu)
+struct gc_xeng_pairs_shape {
+    int kp, nthr, n_blk, per_blk, n_tsplit, ns, grid;
+    long n_items;
+    size_t smem, stage_stride;
+    const void *kern;
+};
+// elements per staged grid row: two spare ones where rows of a multiple of 8
+// would put a column of antennas on one bank
+inline int gc_xeng_pairs_pitch(int L) { return L % 8 == 0 ? L + 2 : L; }
+bool gc_xeng_pairs_eligible(const gc_sel *sel, int vfmt);
+gc_status gc_xeng_pairs_plan(gc_ctx *ctx, const gc_sel *sel, int vfmt, int C, bool autos, gc_xeng_pairs_shape *sh);
+gc_status gc_xeng_pairs_launch(gc_ctx *ctx, const void *volt, int vfmt, int C, int T, const gc_sel *sel,
+                               const gc_xeng_pairs_shape &sh, void *out, void *apart, cudaStream_t s);

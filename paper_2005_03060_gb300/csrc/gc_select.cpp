@@ -85,15 +85,83 @@ void fill_pairs(gc_sel *s) {
         s->type_ptr.push_back((int32_t)s->pair_i.size());
     }
     s->P = (int)s->pair_i.size();
+    // (on a full grid only omnical reads it, and for many types arithmetic is
+    // faster: 12x12 antennas, 264 types, 10.6 against 17.9 ms; 6x6, 60 types,
+    // 4.1 against 3.4 ms)
     const size_t N = (size_t)L * L;
     s->nbr.clear();
-    if (2 * (size_t)s->n_ubl * N <= (16u << 20)) {
+    if ((s->masked || s->n_ubl <= 64) && 2 * (size_t)s->n_ubl * N <= (16u << 20)) {
         s->nbr.assign(2 * (size_t)s->n_ubl * N, -1);
         for (int q = 0; q < s->P; ++q) {
             const int k = s->pair_type[q];
             s->nbr[(size_t)k * N + s->pair_i[q]] = q;
             s->nbr[(size_t)(s->n_ubl + k) * N + s->pair_j[q]] = q;
         }
+    }
+}
+
+// Order a window's pairs for the pair-list X-engine: groups of 16 whose first
+// members, and whose second members, lie at staged positions that differ
+// modulo 16, so that the 8-byte shared-memory reads of a half warp fall on
+// distinct banks.  Pairs of one type keep i - j, so a class (i - j) mod 16 gives
+// whole groups while it holds every j mod 16; the rest is matched across
+// classes, first fit.  (In type order a group spans two grid rows of its type's
+// rectangle and a 32x32 array pays 1.47 reads for each; in this order 1.04.)
+void order_entries(const gc_sel *s, std::vector<int32_t> &q, std::vector<int32_t> &out) {
+    int n[257] = {0}, at[256];
+    const int pad = gc_xeng_pairs_pitch(s->L) - s->L;
+    auto slot = [&](int e) {
+        const int i = s->pair_i[e] + pad * (s->pair_i[e] / s->L), j = s->pair_j[e] + pad * (s->pair_j[e] / s->L);
+        return (((i - j) & 15) << 4) | (j & 15);
+    };
+    for (int e : q) ++n[slot(e) + 1];
+    for (int b = 0; b < 256; ++b) n[b + 1] += n[b];
+    std::copy(n, n + 256, at);
+    std::vector<int32_t> by(q.size());
+    for (int e : q) by[at[slot(e)]++] = e;
+    std::copy(n, n + 256, at);
+    for (int c = 0; c < 16; ++c) {
+        int whole = n[16 * c + 1] - n[16 * c];
+        for (int r = 1; r < 16; ++r) whole = std::min(whole, n[16 * c + r + 1] - n[16 * c + r]);
+        for (int k = 0; k < whole; ++k)
+            for (int r = 0; r < 16; ++r) out.push_back(by[at[16 * c + r]++]);
+    }
+    unsigned has[16] = {0};   // classes left per j mod 16
+    size_t left = 0;
+    for (int c = 0; c < 16; ++c)
+        for (int r = 0; r < 16; ++r) {
+            const int k = n[16 * c + r + 1] - at[16 * c + r];
+            if (k > 0) has[r] |= 1u << c;
+            left += (size_t)k;
+        }
+    auto take = [&](int c, int r) {
+        const int b = 16 * c + r;
+        out.push_back(by[at[b]++]);
+        if (at[b] == n[b + 1]) has[r] &= ~(1u << c);
+        --left;
+    };
+    for (unsigned turn = 0; left > 0; ++turn) {
+        unsigned used = 0;   // i mod 16 taken by this group
+        int got = 0;
+        for (int k = 0; k < 16; ++k) {
+            const int r = (k + (int)turn) & 15;
+            // class c gives i mod 16 = (r + c) mod 16: rotate the free residues
+            const unsigned free16 = ~used & 0xFFFFu;
+            const unsigned m = has[r] & (((free16 | (free16 << 16)) >> r) & 0xFFFFu);
+            if (!m) continue;
+            int c = (int)(turn & 15);   // first class at or after `turn`, for an even use of the classes
+            while (!(m >> c & 1u)) c = (c + 1) & 15;
+            used |= 1u << ((r + c) & 15);
+            take(c, r);
+            ++got;
+        }
+        for (int r = 0; got < 16 && left > 0; r = (r + 1) & 15)   // keep the groups aligned
+            if (has[r]) {
+                int c = 0;
+                while (!(has[r] >> c & 1u)) ++c;
+                take(c, r);
+                ++got;
+            }
     }
 }
 
@@ -133,6 +201,30 @@ void fill_groups(gc_sel *s) {
         ++s->n_windows;
     }
     s->n_groups = (int)s->grp_t0.size();
+    // entry lists of the pair-list X-engine
+    s->wp_entry.clear();
+    s->wp_off.clear();
+    s->wp_t0.clear();
+    s->wp_t1.clear();
+    const int N = s->L * s->L;
+    if (s->n_windows < 2 || N > 25600) return;   // larger grids do not fit its stages in any format
+    s->wp_entry.reserve((size_t)s->P + (size_t)s->n_windows * N);
+    s->wp_off.push_back(0);
+    std::vector<int32_t> win;
+    for (int g = 0; g < s->n_groups; ++g) {
+        if (s->grp_first[g]) {
+            s->wp_t0.push_back(s->grp_t0[g]);
+            s->wp_t1.push_back(s->grp_t1[g]);
+            win.clear();
+        }
+        for (int o = s->grp_off[g]; o < s->grp_off[g + 1]; ++o)
+            for (int q = s->type_ptr[s->grp_types[o]]; q < s->type_ptr[s->grp_types[o] + 1]; ++q) win.push_back(q);
+        if (g + 1 == s->n_groups || s->grp_first[g + 1]) {   // the window's last group
+            order_entries(s, win, s->wp_entry);
+            for (int j = 0; j < N; ++j) s->wp_entry.push_back(s->P + j);
+            s->wp_off.push_back((int32_t)s->wp_entry.size());
+        }
+    }
 }
 
 // Types with at least one pair between occupied points of `mask`, with
@@ -242,8 +334,9 @@ gc_status gc_sel_upload(gc_ctx *ctx, gc_sel *s) {
                                            &s->pair_type, &s->win_t0,   &s->win_t1,    &s->grp_types,
                                            &s->grp_off,  &s->grp_t0,    &s->grp_t1,    &s->grp_first,
                                            &s->grp_win,  &s->nbr,       &s->grp_dymax, &s->mask,
-                                           &s->tree_ant, &s->tree_pair, &s->tree_sign};
-    constexpr int kParts = 19;
+                                           &s->tree_ant, &s->tree_pair, &s->tree_sign, &s->wp_entry,
+                                           &s->wp_off,   &s->wp_t0,     &s->wp_t1};
+    constexpr int kParts = 23;
     size_t total = 0;
     size_t offs[kParts];
     for (int i = 0; i < kParts; ++i) {
@@ -269,7 +362,8 @@ gc_status gc_sel_upload(gc_ctx *ctx, gc_sel *s) {
                        &s->d_pair_type, &s->d_win_t0,   &s->d_win_t1,    &s->d_grp_types,
                        &s->d_grp_off,  &s->d_grp_t0,    &s->d_grp_t1,    &s->d_grp_first,
                        &s->d_grp_win,  &s->d_nbr,       &s->d_grp_dymax, &s->d_mask,
-                       &s->d_tree_ant, &s->d_tree_pair, &s->d_tree_sign};
+                       &s->d_tree_ant, &s->d_tree_pair, &s->d_tree_sign, &s->d_wp_entry,
+                       &s->d_wp_off,   &s->d_wp_t0,     &s->d_wp_t1};
     for (int i = 0; i < kParts; ++i)
         *dst[i] = parts[i]->empty() ? nullptr : reinterpret_cast<int32_t *>(static_cast<char *>(base) + offs[i]);
     s->d_base = base;

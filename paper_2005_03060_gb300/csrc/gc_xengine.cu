@@ -426,6 +426,34 @@ extern "C" gc_status gc_reduce(gc_ctx *ctx, const void *volt, int vfmt, int L, i
         if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "launch xeng_reduce");
         return GC_OK;
     }
+    // several windows (low-cadence): the pair-list form, which writes
+    // V^reduced itself when the windows are not split in time
+    if (gc_xeng_pairs_eligible(sel, vfmt)) {
+        gc_xeng_pairs_shape sh;
+        st = gc_xeng_pairs_plan(ctx, sel, vfmt, C, autos != nullptr, &sh);
+        if (st != GC_OK) return st;
+        const bool direct = sh.n_tsplit == 1;
+        const size_t part_bytes = direct ? 0 : ((size_t)sh.n_tsplit * C * sel->P * sizeof(float2) + 255) / 256 * 256;
+        const size_t apart_bytes = autos ? (size_t)sel->n_windows * sh.n_tsplit * C * N * sizeof(float) : 0;
+        st = gc_scratch_reserve(ctx, part_bytes + apart_bytes + 512);
+        if (st != GC_OK) return st;
+        char *scr = static_cast<char *>(ctx->scratch);
+        void *apart = autos ? scr + part_bytes : nullptr;
+        st = gc_xeng_pairs_launch(ctx, volt, vfmt, C, T, sel, sh, direct ? vreduced : scr, apart, s);
+        if (st != GC_OK) return st;
+        const int Pr = direct ? 0 : sel->P;   // pairs left to sum over slices
+        const size_t work = (size_t)C * Pr + (autos ? (size_t)C * N : 0);
+        if (work == 0) return GC_OK;
+        const int rgrid = (int)std::min<size_t>((work + 255) / 256, (size_t)ctx->sm_count * 8);
+        const int rec = gc_prof_begin(ctx, s, "xeng_reduce");
+        xeng_reduce<<<rgrid, 256, 0, s>>>(reinterpret_cast<const float2 *>(scr), sh.n_tsplit, C, Pr, vfmt, vreduced,
+                                          static_cast<const float *>(apart), sel->n_windows * sh.n_tsplit, N, autos,
+                                          ctx->status_dev);
+        gc_prof_end(ctx, s, rec);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "launch xeng_reduce");
+        return GC_OK;
+    }
     const int esz = vfmt == GC_C64 ? 8 : (vfmt == GC_C32H ? 4 : 1);
     const size_t sample_bytes = (size_t)N * esz;
     const bool tma = gc_aligned(volt, 16) && sample_bytes % 16 == 0;
