@@ -275,9 +275,12 @@ GC_API gc_status gc_quantize(gc_ctx *ctx, const float *volt, int C, int T, int N
  * pair's window length) and the model V_p ~ g_i conj(g_j) V_alpha(p) is
  * fitted by least squares with uniform weights (Eq. noisecov):
  *   GC_LINCAL  Gauss-Newton on (Re, Im) of every gain and model visibility;
- *              banded normal equations (antennas row-major), FP64 (GC_FP64)
- *              or FP32 (GC_FP32); the four degeneracies are projected out
- *              of each step; up to 64 baseline-types (subset selections).
+ *              residuals, gradient, chi^2 and the state in FP64 (GC_FP64) or
+ *              FP32 (GC_FP32); the step from banded normal equations
+ *              (antennas row-major) factorised in FP32, with a pass of
+ *              iterative refinement in FP64 while steps are large; the four
+ *              degeneracies are projected out of each step; up to 64
+ *              baseline-types (subset selections).
  *   GC_OMNICAL damped simultaneous least-squares fixed point (damping 0.3
  *              by default, Sec. 3), FP32; any selection (low-cadence).
  *   GC_LINCAL_CG Gauss-Newton with the step from conjugate gradients on
