@@ -15,6 +15,7 @@ struct CalParams {
     int ax, ay;                  // indices of types (1,0) and (0,1)
     int stencil;                 // matrix-free operator by per-antenna gather (<= kStencilTypes types)
     int st_halo;                 // largest |dx| or |dy| of a type (stencil operator)
+    int dense;                   // matrix-free operator as lag-plane correlations (selections of many types)
     // partly occupied lattice (null / L*L otherwise): occupancy [N], the
     // breadth-first start-point tree over the axis types, antennas
     const int32_t *mask, *tree_ant, *tree_pair, *tree_sign;

@@ -29,6 +29,7 @@ constexpr int kStencilTypes = 16; // baseline-types the stencil operator holds i
 // them in global memory (L2) at two CTAs per SM -- measured faster than one
 // CTA per SM with a larger arena (the solver is latency-bound).
 constexpr size_t kCgSmemMax = 100u * 1024u;
+constexpr size_t kCgDnSmem = 215u * 1024u;   // lag-plane operator, one CTA per SM
 constexpr int kMaxUbl = 64;   // baseline-types the direct solver (gc_lincal.cu) takes
 
 // State of a Gauss-Newton step's projection (pair-list solver).
@@ -118,6 +119,12 @@ struct CgWork {
     float *G, *D;
     unsigned short *cid;
     int coarse_gather;       // every type offset within one patch side: gather assembly
+    // lag-plane operator (see dense_op_pass), shared memory
+    float *U;                // [2L-1][2L-1] |V|^2 per lag, both signs
+    float2 *Q;               // [2L-1][2L-1] |V|^2 w per lag (conjugate at the opposite lag)
+    float2 *Ea;              // [L][3L+5] G q, zero off the grid
+    float *Eg;               // [L][3L+5] G
+    float2 *yb, *zb;         // sums per antenna [N], per lag [L][lag row]
     int n, m;
     int B, npx, ncp, nc, cv; // patch side, patches per row, patches, coarse size, V in coarse space
 };
@@ -785,6 +792,287 @@ __device__ float rel_chi2(const CalParams &p, int c, const float *tg, const floa
     return s[0];
 }
 
+// ---- Lag-plane operator, for selections that hold a good part of all pairs
+// (low-cadence calibration takes every type).  In relative coordinates the
+// weights factor as W_ij = G_i G_j U(i - j) with U(d) = |V_d|^2, so the sums
+// over pairs are 2-D correlations over the grid,
+//   (A q)_i = D_i q_i + G_i sum_j [U(i - j) conj(G_j q_j) + Q(i - j) G_j],
+//   (A q)_k = D_k w_k + U_k sum_j [G_i q_i G_j + G_i conj(G_j q_j)],  i = j + d_k,
+// with Q(d_k) = U_k w_k, Q(-d_k) = conj(Q(d_k)) and U = Q = 0 for types outside
+// the selection: dense sums of L^4 terms without pair lists, indices or
+// atomics.  A thread keeps eight neighbouring outputs and slides a window of
+// eight plane values along a grid row, so a step of 32 multiply-adds reads one
+// new plane value and one broadcast antenna.  What bounds it is FP32 issue:
+// 24x24 antennas (331 776 terms, 165 600 pairs) take about 20 us a pass, the
+// scatter over the pair list 240 us; 64 channels of that array calibrate in
+// 4.5 ms, 40.9 ms with the scatter.
+constexpr int kCgDnThreads = 512;
+__host__ __device__ inline int dense_lag_row(int L) { return (2 * L - 1 + 7) / 8 * 8; }
+__host__ __device__ inline int dense_row(int L) { return 3 * L + 5; }
+__host__ __device__ inline size_t cg_dense_floats(int L) {
+    const size_t W = 2 * L - 1, plane = (W * W + 8 + 3) / 4 * 4, E = ((size_t)L * dense_row(L) + 3) / 4 * 4;
+    return plane + 2 * plane + 2 * E + E + 2 * (((size_t)L * L + 1) / 2 * 2) + 2 * (size_t)L * dense_lag_row(L);
+}
+__device__ void dense_layout(const CalParams &p, CgWork &w, float *at) {
+    const int L = p.L;
+    const size_t W = 2 * L - 1, plane = (W * W + 8 + 3) / 4 * 4, E = ((size_t)L * dense_row(L) + 3) / 4 * 4;
+    w.U = at;
+    w.Q = reinterpret_cast<float2 *>(at + plane);
+    w.Ea = reinterpret_cast<float2 *>(at + 3 * plane);
+    w.Eg = at + 3 * plane + 2 * E;
+    w.yb = reinterpret_cast<float2 *>(at + 3 * plane + 3 * E);
+    w.zb = w.yb + ((size_t)L * L + 1) / 2 * 2;
+}
+
+// yb_i = sum_j U(i - j) conj(a_j) + Q(i - j) G_j over the whole grid (a, G in Ea, Eg)
+__device__ void dense_antenna_sums(const CalParams &p, const CgWork &w) {
+    const int L = p.L, W = 2 * L - 1, Ew = dense_row(L);
+    const int nseg = (L + 7) / 8, tasks = L * nseg, S = min(L, max(1, (int)blockDim.x / tasks));
+    // (tasks <= blockDim.x: L <= 64)
+    const int task = threadIdx.x % tasks, split = threadIdx.x / tasks;
+    const int y = task / nseg, x0 = 8 * (task - y * nseg);
+    float2 acc[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc[u] = make_float2(0.f, 0.f);
+    if (split < S) {
+        for (int jy = split * L / S; jy < (split + 1) * L / S; ++jy) {
+            const float *pu = w.U + (y - jy + L - 1) * W + x0 + L - 1;
+            const float2 *pq = w.Q + (y - jy + L - 1) * W + x0 + L - 1;
+            const float2 *ea = w.Ea + jy * Ew + L - 1;
+            const float *eg = w.Eg + jy * Ew + L - 1;
+            // output u at step jx uses the plane value u - jx, in slot (u - jx) & 7
+            float U[8];
+            float2 Q[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                U[u] = pu[u];
+                Q[u] = pq[u];
+            }
+            for (int j0 = 0; j0 < L; j0 += 8) {
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                    const int jx = j0 + v;
+                    if (jx < L) {
+                        if (jx > 0) {
+                            U[(8 - v) & 7] = pu[-jx];
+                            Q[(8 - v) & 7] = pq[-jx];
+                        }
+                        const float2 a = ea[jx];
+                        const float g = eg[jx];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const int s = (u - v) & 7;
+                            acc[u].x = fmaf(U[s], a.x, fmaf(Q[s].x, g, acc[u].x));
+                            acc[u].y = fmaf(-U[s], a.y, fmaf(Q[s].y, g, acc[u].y));
+                        }
+                    }
+                }
+            }
+        }
+    }
+    // the row splits are added in turn (a fixed order)
+    for (int s = 0; s < S; ++s) {
+        if (split == s) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (x0 + u < L) {
+                    float2 &o = w.yb[y * L + x0 + u];
+                    o = s == 0 ? acc[u] : make_float2(o.x + acc[u].x, o.y + acc[u].y);
+                }
+        }
+        __syncthreads();
+    }
+}
+
+// zb(d) = sum_j a_i G_j + G_i conj(a_j), i = j + d, for the lags with d_y >= 0
+__device__ void dense_lag_sums(const CalParams &p, const CgWork &w) {
+    const int L = p.L, Ew = dense_row(L), Wz = dense_lag_row(L);
+    // a task takes the lag rows h and L - h, together L rows of j
+    const int nseg = Wz / 8, nh = L / 2 + 1, tasks = nh * nseg, S = min(L, max(1, (int)blockDim.x / tasks));
+    const int task = threadIdx.x % tasks, split = threadIdx.x / tasks;
+    const int h = task / nseg, e0 = 8 * (task - h * nseg);
+    const int dyb = h > 0 && 2 * h != L ? L - h : -1, rows = dyb < 0 ? L - h : L;
+    float2 acc[2][8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc[0][u] = acc[1][u] = make_float2(0.f, 0.f);
+    if (split < S) {
+        const int r1 = min(rows, (split + 1) * L / S);
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+            const int dy = part == 0 ? h : dyb, off = part == 0 ? 0 : L - h;
+            const int lo = max(split * L / S, off), hi = part == 0 ? min(r1, L - h) : (dyb < 0 ? 0 : r1);
+            for (int r = lo; r < hi; ++r) {
+                const int jy = r - off;
+                const float2 *ei = w.Ea + (jy + dy) * Ew + e0, *ej = w.Ea + jy * Ew + L - 1;
+                const float *gi = w.Eg + (jy + dy) * Ew + e0, *gj = w.Eg + jy * Ew + L - 1;
+                // lag u at step jx uses the antenna u + jx, in slot (u + jx) & 7
+                float2 A[8];
+                float G[8];
+#pragma unroll
+                for (int u = 0; u < 7; ++u) {
+                    A[u] = ei[u];
+                    G[u] = gi[u];
+                }
+                for (int j0 = 0; j0 < L; j0 += 8) {
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) {
+                        const int jx = j0 + v;
+                        if (jx < L) {
+                            A[(v + 7) & 7] = ei[jx + 7];
+                            G[(v + 7) & 7] = gi[jx + 7];
+                            const float2 b = ej[jx];
+                            const float g = gj[jx];
+#pragma unroll
+                            for (int u = 0; u < 8; ++u) {
+                                const int s = (u + v) & 7;
+                                acc[part][u].x = fmaf(A[s].x, g, fmaf(G[s], b.x, acc[part][u].x));
+                                acc[part][u].y = fmaf(A[s].y, g, fmaf(-G[s], b.y, acc[part][u].y));
+                            }
+                        }
+                    }
+                }
+            }
+        }
+    }
+    for (int s = 0; s < S; ++s) {
+        if (split == s) {
+#pragma unroll
+            for (int part = 0; part < 2; ++part) {
+                const int dy = part == 0 ? h : dyb;
+                if (dy < 0 || dy >= L) continue;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    float2 &o = w.zb[dy * Wz + e0 + u];
+                    o = s == 0 ? acc[part][u]
+                               : make_float2(o.x + acc[part][u].x, o.y + acc[part][u].y);
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// acc = A q; returns this thread's part of q.(A q + mu G q) (as rel_op_pass).
+__device__ float dense_op_pass(const CalParams &p, const CgWork &w, float mu) {
+    const int L = p.L, N = p.N, K = p.n_ubl, W = 2 * L - 1, Ew = dense_row(L), Wz = dense_lag_row(L);
+    const float2 *q = reinterpret_cast<const float2 *>(w.pp);
+    float2 *out = reinterpret_cast<float2 *>(w.acc);
+    for (int m = threadIdx.x; m < N; m += blockDim.x) {
+        const int y = m / L, x = m - y * L;
+        const float g = w.G[m];
+        w.Ea[y * Ew + L - 1 + x] = make_float2(g * q[m].x, g * q[m].y);
+    }
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1), o = (dy + L - 1) * W + dx + L - 1;
+        const float u = w.G[N + k];
+        const float2 t = make_float2(u * q[N + k].x, u * q[N + k].y);
+        w.Q[o] = t;
+        w.Q[W * W - 1 - o] = make_float2(t.x, -t.y);
+    }
+    __syncthreads();
+    dense_antenna_sums(p, w);
+    dense_lag_sums(p, w);
+    float curv = 0.f;
+    for (int m = threadIdx.x; m < N; m += blockDim.x) {
+        const float2 v = q[m], s = w.yb[m];
+        const float D = w.D[m], G = w.G[m], mg = mu * G;
+        const float2 o = make_float2(fmaf(D, v.x, G * s.x), fmaf(D, v.y, G * s.y));
+        out[m] = o;
+        curv = fmaf(v.x, o.x + mg * v.x, fmaf(v.y, o.y + mg * v.y, curv));
+    }
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1);
+        const float2 v = q[N + k], s = w.zb[dy * Wz + dx + L - 1];
+        const float D = w.D[N + k], U = w.G[N + k], mg = mu * U;
+        const float2 o = make_float2(fmaf(D, v.x, U * s.x), fmaf(D, v.y, U * s.y));
+        out[N + k] = o;
+        curv = fmaf(v.x, o.x + mg * v.x, fmaf(v.y, o.y + mg * v.y, curv));
+    }
+    return curv;
+}
+
+// Residual pass of the lag-plane form (same results as rel_resid_pass): a warp
+// per type over its pairs, h = conj(m) r added to both members (shared-memory
+// atomics: consecutive pairs touch consecutive antennas) and summed per type;
+// the antennas' diagonals by a correlation.
+__device__ double dense_resid_pass(const CalParams &p, int c, const CgWork &w, bool staged, double *red, float *dmax) {
+    const int L = p.L, N = p.N, K = p.n_ubl, W = 2 * L - 1, Ew = dense_row(L);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float2 *xg = reinterpret_cast<float2 *>(w.pp);
+    const float *xv = staged ? w.pp + 2 * N : w.xv;
+    for (int m = threadIdx.x; m < N; m += blockDim.x) {
+        const float2 g = staged ? xg[m] : reinterpret_cast<const float2 *>(w.xg)[m];
+        if (!staged) xg[m] = g;
+        const int y = m / L, x = m - y * L;
+        const float G = g.x * g.x + g.y * g.y;
+        w.G[m] = G;
+        w.Eg[y * Ew + L - 1 + x] = G;
+        w.Ea[y * Ew + L - 1 + x] = make_float2(G, 0.f);
+        w.yb[m] = make_float2(0.f, 0.f);
+    }
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+        const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1), o = (dy + L - 1) * W + dx + L - 1;
+        const float u = xv[2 * k] * xv[2 * k] + xv[2 * k + 1] * xv[2 * k + 1];
+        w.U[o] = w.U[W * W - 1 - o] = u;
+        w.Q[o] = w.Q[W * W - 1 - o] = make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    float chi = 0.f;
+    const float2 *vf = reinterpret_cast<const float2 *>(p.vred) + (size_t)c * p.P;
+    const int2 *vi = reinterpret_cast<const int2 *>(p.vred) + (size_t)c * p.P;
+    float *hb = reinterpret_cast<float *>(w.yb);
+    for (int k = wp; k < K; k += nw) {
+        const float inv = 1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
+        const float Vx = xv[2 * k], Vy = xv[2 * k + 1];
+        float tx = 0.f, ty = 0.f, td = 0.f;
+        const int q1 = __ldg(p.type_ptr + k + 1);
+        for (int q = __ldg(p.type_ptr + k) + lane; q < q1; q += 32) {
+            const int i = __ldg(p.pair_i + q), j = __ldg(p.pair_j + q);
+            float2 o;
+            if (p.vfmt == GC_C64) {
+                o = vf[q];
+            } else {
+                const int2 v = vi[q];
+                o = make_float2((float)v.x, (float)v.y);
+            }
+            const float2 gi = xg[i], gj = xg[j];
+            const float ex = gi.x * gj.x + gi.y * gj.y, ey = gi.y * gj.x - gi.x * gj.y;
+            const float mx = ex * Vx - ey * Vy, my = ex * Vy + ey * Vx;
+            const float rx = o.x * inv - mx, ry = o.y * inv - my;
+            chi = fmaf(rx, rx, fmaf(ry, ry, chi));
+            const float hx = mx * rx + my * ry, hy = mx * ry - my * rx;
+            tx += hx;
+            ty += hy;
+            td += mx * mx + my * my;
+            atomicAdd(&hb[2 * i], hx);
+            atomicAdd(&hb[2 * i + 1], hy);
+            atomicAdd(&hb[2 * j], hx);
+            atomicAdd(&hb[2 * j + 1], -hy);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            tx += __shfl_xor_sync(0xffffffffu, tx, o);
+            ty += __shfl_xor_sync(0xffffffffu, ty, o);
+            td += __shfl_xor_sync(0xffffffffu, td, o);
+        }
+        if (lane == 0) {
+            w.acc[2 * (N + k)] = tx;
+            w.acc[2 * (N + k) + 1] = ty;
+            w.D[N + k] = td;
+        }
+    }
+    __syncthreads();
+    for (int m = threadIdx.x; m < N; m += blockDim.x) reinterpret_cast<float2 *>(w.acc)[m] = w.yb[m];
+    __syncthreads();
+    dense_antenna_sums(p, w);
+    float dm = 0.f;
+    for (int m = threadIdx.x; m < N; m += blockDim.x) {
+        const float s = w.yb[m].x;
+        w.D[m] = w.G[m] * s;
+        if (w.G[m] > 0.f) dm = fmaxf(dm, s);
+    }
+    return rel_resid_finish(p, w, xv, red, dmax, chi, dm);
+}
+
 // Two-level preconditioner.  The coarse space scales each patch of B x B
 // antennas by one complex factor and (when there are few types) each model
 // visibility by another: dg_i = g_i c_P(i), dV_k = V_k c_k.  For a pair, J
@@ -1012,6 +1300,30 @@ __device__ void coarse_assemble_gather(const CalParams &p, const CgWork &w, floa
     __syncthreads();
 }
 
+// Assembly from the factored weights W_ij = G_i G_j U(i - j) (lag-plane form,
+// no model visibilities in the coarse space): entry (a, b) is the sum of W
+// over antennas of patch a and of patch b.
+__device__ void coarse_assemble_dense(const CalParams &p, const CgWork &w, float mu) {
+    const int nc = w.nc, L = p.L, B = w.B, npx = w.npx, W = 2 * L - 1;
+    for (int t = threadIdx.x; t < nc * nc; t += blockDim.x) {
+        const int a = t / nc, b = t - a * nc;
+        const int ax = a % npx * B, ay = a / npx * B, bx = b % npx * B, by = b / npx * B;
+        float s = 0.f, d = 0.f;
+        for (int iy = ay; iy < min(L, ay + B); ++iy)
+            for (int ix = ax; ix < min(L, ax + B); ++ix) {
+                const float *u = w.U + (iy + L - 1) * W + ix + L - 1;
+                float r = 0.f;
+                for (int jy = by; jy < min(L, by + B); ++jy)
+                    for (int jx = bx; jx < min(L, bx + B); ++jx) r = fmaf(u[-jy * W - jx], w.G[jy * L + jx], r);
+                s = fmaf(w.G[iy * L + ix], r, s);
+                d += w.D[iy * L + ix] + mu * w.G[iy * L + ix];
+            }
+        w.Ca[t] = a == b ? d + s : s;
+        w.Cp[t] = a == b ? d - s : -s;
+    }
+    __syncthreads();
+}
+
 // Block-wide max / sum of one float (all threads get the result).
 __device__ __forceinline__ float block_allreduce(float v, bool is_max, float *buf /* [32] */) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -1091,6 +1403,7 @@ __device__ void coarse_invert(float *A, int nc, int ncp, bool amp, bool cv, floa
 __device__ void cg_coarse_setup(const CalParams &p, const CgWork &w, float mu) {
     __shared__ float s_buf[32];
     if (p.stencil && w.coarse_gather) coarse_assemble_gather(p, w, mu);
+    else if (p.dense && !w.cv) coarse_assemble_dense(p, w, mu);
     else coarse_assemble_scatter(p, w, mu);
     const int nn = w.nc * w.nc;
     for (int m = 0; m < 2; ++m) {
@@ -1314,11 +1627,13 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
 }
 
 // One channel of matrix-free Gauss-Newton in relative coordinates (the
-// stencil operator; see rel_op_pass).  Same outer iteration, forcing terms,
+// stencil operator, see rel_op_pass, or with kDense the lag-plane operator,
+// see dense_op_pass).  Same outer iteration, forcing terms,
 // preconditioner, projection, line search and stopping rule as
 // cg_solve_channel; the CG vectors hold (q, w) and the search direction q
 // lives in shared memory beside G, D and the coarse indices.  Convergence
 // tests use the (g, V)-form norms, |r|^2 / G per element.
+template <bool kDense>
 __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, double cg_tol, int cg_max, double *red,
                                      float *redf) {
     const int ne = p.N + p.n_ubl, L = p.L, nc = w.nc, N = p.N;
@@ -1328,7 +1643,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
     const uint64_t t_start = gc_globaltimer();
     if (p.warm) {
         for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            const float2 g = p.gains[(size_t)c * N + i];
+            const float2 g = !kDense || !p.mask || p.mask[i] ? p.gains[(size_t)c * N + i] : make_float2(0.f, 0.f);
             w.xg[2 * i] = g.x;
             w.xg[2 * i + 1] = g.y;
         }
@@ -1370,11 +1685,13 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
             // the preconditioner's diagonal and the norm's weights by the
             // fast reciprocal (within 2 ulp; a preconditioner only has to be
             // the same operator at every step, which this is)
-            const float iv = __fdividef(1.f, w.D[e] + mu * w.G[e]);
+            // (empty points of a partly occupied lattice: G = D = r = 0)
+            const float Ge = w.G[e], dg = w.D[e] + mu * Ge;
+            const float iv = !kDense || dg > 0.f ? __fdividef(1.f, dg) : 0.f;
             const float2 z = make_float2(r.x * iv, r.y * iv);
             zs[e] = z;
             rzj = fmaf(r.x, z.x, fmaf(r.y, z.y, rzj));
-            rr += __fdividef(r.x * r.x + r.y * r.y, w.G[e]);
+            if (!kDense || Ge > 0.f) rr += __fdividef(r.x * r.x + r.y * r.y, Ge);
             const unsigned cu = w.cid[e];
             ci = cu == 0xffffu ? -1 : (int)cu;
         }
@@ -1488,7 +1805,8 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
         // tried with chi^2 alone.  (One call site keeps one copy of the
         // pass in the instruction stream.)
         float dmax = 0.f;
-        const double c2 = rel_resid_pass(p, c, w, staged, red, &dmax);
+        const double c2 = kDense ? dense_resid_pass(p, c, w, staged, red, &dmax)
+                                 : rel_resid_pass(p, c, w, staged, red, &dmax);
         if (staged) {
             staged = false;
             const bool full = c2 <= chi2 * (1.0 + 1e-6) + 1e-30;
@@ -1502,8 +1820,8 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
                     stage[e] = make_float2(sv.x + step * dp.x, sv.y + step * dp.y);
                 }
                 __syncthreads();
-                const float ch = rel_chi2(p, c, reinterpret_cast<const float *>(stage),
-                                          reinterpret_cast<const float *>(stage + N), redf);
+                const float *sg = reinterpret_cast<const float *>(stage);
+                const float ch = kDense ? chi2_of<float>(p, c, sg, sg + 2 * N, redf) : rel_chi2(p, c, sg, sg + 2 * N, redf);
                 if ((double)ch <= chi2 * (1.0 + 1e-6) + 1e-30 || ls == 7) break;
             }
             for (int e = threadIdx.x; e < ne; e += blockDim.x) {
@@ -1558,7 +1876,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
             (float)fmin(0.05, fmax(cg_tol, sqrt(sqrt(sqrt((double)bnorm2 / fmax(grad0, 1e-300))))));
         for (int k = 0; k < cg_max && bnorm2 > 0.f; ++k) {
             ++inner;
-            float v1[1] = {rel_op_pass(p, w, mu)};   // acc = A q; q.(A + mu G) q
+            float v1[1] = {kDense ? dense_op_pass(p, w, mu) : rel_op_pass(p, w, mu)};   // acc = A q; q.(A + mu G) q
             fast_sum<1>(v1, sbuf, par);
             if (!(v1[0] > 0.f)) break;
             const float alpha = rz / v1[0];
@@ -1707,11 +2025,38 @@ lincal_cg_kernel(const CalParams p, double cg_tol, int cg_max, int smem_floats) 
         if (c >= p.C) break;
         if constexpr (kSten) {
             if (p.stencil) {
-                cg_solve_channel_rel(p, c, w, cg_tol, cg_max, red, redf);
+                cg_solve_channel_rel<false>(p, c, w, cg_tol, cg_max, red, redf);
                 continue;
             }
         }
         cg_solve_channel<kPipe>(p, c, w, cg_tol, cg_max, red, redf);
+    }
+}
+
+// The lag-plane operator (p.dense set): one CTA per SM, everything that the
+// operator reads in shared memory.
+__global__ void __launch_bounds__(kCgDnThreads, 1)
+lincal_cg_dense(const CalParams p, double cg_tol, int cg_max, int smem_floats, int coarse_smem) {
+    __shared__ double red[32 * 14];
+    __shared__ float redf[32 * 14];
+    __shared__ float s_rc[2 * kMaxCoarse], s_yc[2 * kMaxCoarse];
+    extern __shared__ __align__(16) float arena[];
+    __shared__ int s_item;
+    const int dn = (int)cg_dense_floats(p.L);
+    CgWork w = cg_layout(p, p.work + (size_t)blockIdx.x * p.work_per_cta, arena + dn, smem_floats - dn, 3,
+                         coarse_smem != 0);
+    w.rc = s_rc;
+    w.yc = s_yc;
+    dense_layout(p, w, arena);
+    for (int i = threadIdx.x; i < dn; i += blockDim.x) arena[i] = 0.f;   // what lies off the grid and absent types stay 0
+    __syncthreads();
+    for (;;) {
+        if (threadIdx.x == 0) s_item = (int)atomicAdd(p.counter, 1u);
+        __syncthreads();
+        const int c = s_item;
+        __syncthreads();
+        if (c >= p.C) break;
+        cg_solve_channel_rel<true>(p, c, w, cg_tol, cg_max, red, redf);
     }
 }
 
@@ -1758,7 +2103,7 @@ lincal_cg_batched(const __grid_constant__ BatchParams bp) {
         w.yc = s_yc;
         if constexpr (kSten) {
             if (p.stencil) {
-                cg_solve_channel_rel(p, item - bp.prefix[slot], w, bp.cg_tol, bp.cg_max, red, redf);
+                cg_solve_channel_rel<false>(p, item - bp.prefix[slot], w, bp.cg_tol, bp.cg_max, red, redf);
                 continue;
             }
         }
@@ -1920,6 +2265,14 @@ static gc_status fill_params(gc_ctx *ctx, gc_sel *sel, int C, const void *vreduc
     // both full-grid selection builders take baseline-types whole, in
     // pair_index order; a partly occupied lattice takes the pair-list form
     p.stencil = ctx->tune[GC_TUNE_CAL_OP] == 0 && sel->n_ubl <= kStencilTypes && !sel->masked ? 1 : 0;
+    // the lag planes: many types, at least a sixteenth of all pairs (the pair
+    // scatter costs 2.9 cycles a pair and SM, the planes 0.08 a product of
+    // antennas: the lines cross at a thirty-eighth), and planes that fit beside the vectors
+    const size_t dn = (cg_dense_floats(sel->L) + cg_sten_floats(p.N, p.n_ubl)) * sizeof(float);
+    p.dense = o.solver == GC_LINCAL_CG && ctx->tune[GC_TUNE_CAL_OP] == 0 && !p.stencil && sel->L <= 64 &&
+                      16.0 * sel->P >= (double)p.N * p.N && dn <= kCgDnSmem
+                  ? 1
+                  : 0;
     p.st_halo = 0;
     for (int k = 0; k < sel->n_ubl; ++k)
         p.st_halo = std::max(p.st_halo, std::max(std::abs(sel->types[2 * k]), std::abs(sel->types[2 * k + 1])));
@@ -1978,6 +2331,7 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     int occ = 0;
     size_t per_cta, cg_smem = 0;
     bool pipe = false;
+    int dense_coarse = 0;
     const void *kfn;
     if (o.solver == GC_LINCAL) {
         if (sel->n_ubl > kMaxUbl)
@@ -1988,6 +2342,16 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     }
     if (o.solver == GC_LINCAL_CG) {
         per_cta = cg_bytes(p.N, p.n_ubl, p.P);
+        if (p.dense) {
+            kfn = (const void *)lincal_cg_dense;
+            e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgDnSmem);
+            if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(lincal_cg_dense)");
+            cg_smem = (cg_dense_floats(p.L) + cg_sten_floats(p.N, p.n_ubl)) * sizeof(float);
+            const size_t cf = cg_coarse_floats(p.L, p.n_ubl) * sizeof(float);
+            dense_coarse = cg_smem + cf <= kCgDnSmem ? 1 : 0;
+            if (dense_coarse) cg_smem += cf;
+            else if (cg_smem + cf / 2 <= kCgDnSmem) cg_smem += cf / 2;   // one system: the inversion's scratch
+        } else {
         cg_smem = cg_arena_bytes(p.N, p.n_ubl, p.L, kCgSmemMax, p.stencil != 0);
         // pair-scatter operator with its hot vectors in global memory: the pipelined pass
         pipe = !p.stencil && cg_hot_floats(p.N, p.n_ubl, false) * sizeof(float) > cg_smem;
@@ -1996,12 +2360,13 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
                                 : (const void *)lincal_cg_kernel<false, false>);
         e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
         if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(lincal_cg)");
+        }
     } else {
         per_cta = sizeof(float) * (size_t)(2 * p.N + 2 * p.n_ubl + p.N + 2 * p.N + 2 * p.n_ubl + 64);
         kfn = (const void *)omnical_kernel;
     }
     per_cta = (per_cta + 255) & ~size_t(255);
-    const int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? kCgStThreads : kCgThreads) : kCThreads;
+    const int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? kCgStThreads : (p.dense ? kCgDnThreads : kCgThreads)) : kCThreads;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, nthr, cg_smem);
     if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(calibration)");
     if (ctx->tune[GC_TUNE_CAL_CTAS] > 0) occ = std::min(occ, ctx->tune[GC_TUNE_CAL_CTAS]);
@@ -2020,6 +2385,7 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     if (o.solver == GC_LINCAL_CG) {
         const int sf = (int)(cg_smem / sizeof(float));
         if (p.stencil) lincal_cg_kernel<false, true><<<grid, kCgStThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
+        else if (p.dense) lincal_cg_dense<<<grid, kCgDnThreads, cg_smem, s>>>(p, 1e-4, 500, sf, dense_coarse);
         else if (!pipe) lincal_cg_kernel<false, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
         else lincal_cg_kernel<true, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
     } else {
@@ -2050,6 +2416,7 @@ extern "C" gc_status gc_calibrate_batched(gc_ctx *ctx, int n_arrays, const gc_ba
         gc_status st = fill_params(ctx, const_cast<gc_sel *>(it.sel), it.C, it.vreduced, it.vfmt, it.autos, o,
                                    it.gains, it.vmodel, it.stats, bp.arr[a]);
         if (st != GC_OK) return st;
+        bp.arr[a].dense = 0;   // (the batched kernel holds the other two operators)
         per_cta = std::max(per_cta, cg_bytes(bp.arr[a].N, bp.arr[a].n_ubl, bp.arr[a].P));
         cost.push_back({(double)bp.arr[a].P + 4.0 * bp.arr[a].N, a});
     }
