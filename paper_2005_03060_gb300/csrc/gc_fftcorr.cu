@@ -26,6 +26,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <vector>
 
@@ -35,7 +36,7 @@
 namespace {
 
 // ----------------------------------------------------------------- config
-template <int M_, int R_, int F1_, int F2_, int NT_, int G_, int VF_, int MINB_ = 1>
+template <int M_, int R_, int F1_, int F2_, int NT_, int G_, int VF_, int MINB_ = 1, int NST_ = 2, int QG_ = 1, int CH_ = 0>
 struct Cfg {
     static constexpr int M = M_, R = R_, F1 = F1_, F2 = F2_, NT = NT_, G = G_, VF = VF_;
     static constexpr int MINB = MINB_;                  // resident CTAs per SM the registers must allow
@@ -46,7 +47,12 @@ struct Cfg {
     static constexpr int S2 = M / F2;                   // column residues
     static constexpr int J2 = (LMAX + F2 - 1) / F2;     // column folds
     static constexpr int NCOL = MX * S2;                // column items per group
-    static constexpr int NTHREADS = G * NCOL;
+    // CTAs per SM that the time chunks are sized for (0: those that are resident): fixed where a launch shape
+    // was changed, so that the chunks, and with them the rounding of the FP32 sums, stay what they were
+    static constexpr int CHUNK_CTAS = CH_;
+    static constexpr int QG = QG_;                      // k_x residues a CTA works on side by side
+    static constexpr int GTHREADS = G * NCOL;           // threads per residue
+    static constexpr int NTHREADS = QG * GTHREADS;
     static constexpr int GNT = G * NT;                  // samples per iteration
     static constexpr int ESZ = VF == GC_C64 ? 8 : (VF == GC_C32H ? 4 : 1);   // bytes per antenna-sample
     // padded stage row (bytes): the smallest odd number of 16-byte units
@@ -54,19 +60,24 @@ struct Cfg {
     static constexpr int ROWU = (LMAX * ESZ + 15) / 16;
     static constexpr int ROWB = 16 * (ROWU % 2 == 1 ? ROWU : ROWU + 1);
     static constexpr int ROWE = ROWB / ESZ;             // elements per stage row
-    static constexpr int CROW = LMAX + 2;               // coefficient row (float2)
+    // coefficient row (float2): complex64 and binary16 rows read 16 bytes (two
+    // antennas) at a time, 4+4-bit rows 8, on an odd pitch, so that the rows of
+    // consecutive lanes fall on distinct banks (an even one: two-way conflicts)
+    static constexpr int CROW = VF == GC_I4C ? LMAX + 1 : LMAX + 2;
     static constexpr int IROW = MX + 1;                 // intermediate row (float2)
     static constexpr int STAGE_BYTES = GNT * LMAX * ROWB;
-    static constexpr int NSTAGE = 2;
+    static constexpr int NSTAGE = NST_;
     // shared memory layout (bytes)
     static constexpr int OFF_BAR = 0;
     static constexpr int OFF_TW = 128;
     static constexpr int OFF_COEF = OFF_TW + ((M * 8 + 127) / 128) * 128;
     static constexpr int OFF_STAGE = OFF_COEF + ((LMAX * CROW * 8 + 127) / 128) * 128;
     static constexpr int OFF_INTER = OFF_STAGE + NSTAGE * ((STAGE_BYTES + 127) / 128) * 128;
-    static constexpr int SMEM = OFF_INTER + GNT * LMAX * IROW * 8;
+    static constexpr int INTER = GNT * LMAX * IROW;     // intermediate of one residue (float2)
+    static constexpr int SMEM = OFF_INTER + QG * INTER * 8;
     static_assert(MX % F1 == 0 && M % F2 == 0, "bad FFT split");
     static_assert(ROWB % 16 == 0 && (ROWB / 16) % 2 == 1, "stage row must be an odd number of 16B");
+    static_assert(R % QG == 0 && (QG == 1 || S1 > 1), "residues of one CTA share the coefficients");
     static_assert(F1 % 4 == 0 && (VF != GC_I4C || F1 % 16 == 0 || LMAX <= 16), "row reads");
     static_assert((G - 1) * NCOL * F2 * 4 <= GNT * LMAX * IROW * 8, "group partial spectra must fit the intermediate");
 };
@@ -79,7 +90,7 @@ struct Params {
     int L, C, T;
     int chunk_len;           // multiple of G*NT
     int n_chunks;
-    int n_items;             // C * R * n_chunks
+    int n_items;             // C * (R / QG) * n_chunks
     const unsigned char *mask = nullptr;   // [L*L] occupied lattice points, or null (all)
 };
 
@@ -156,16 +167,55 @@ __device__ __forceinline__ void col_fold2(float2 (&b)[K::F2], const float2 *icol
     }
 }
 
-template <class K, bool kTMA>
-__global__ void __launch_bounds__(K::NTHREADS, K::MINB)
+// How voltages reach the stage: plain loads; tiled copies, which also make the
+// zero padding (grid rows of whole 16-byte units); or bulk copies of the
+// samples as they lie in memory into the second stage's space, repacked into
+// padded rows from there (any other row length: plain loads leave their
+// latency in every iteration; 331 antennas on 21x21 points, binary16, 128
+// channels of 2047 samples: 2.46 ms, 2.16 ms with bulk copies).
+enum { kStagePlain = 0, kStageTiled = 1, kStageBulk = 2 };
+
+// Padded rows of the samples at t from their bytes in `raw` (first byte at raw[off]).
+template <class K>
+__device__ void repack_rows(const Params &p, unsigned char *stage, const unsigned char *raw, int off, int t) {
+    const int L = p.L, lane = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < K::GNT * L; r += K::NTHREADS / 32) {
+        const int u = r / L, y = r - u * L;
+        const bool ok = t + u < p.T;
+        unsigned char *dst = stage + (u * K::LMAX + y) * K::ROWB;
+        const unsigned char *src = raw + off + (u * L + y) * L * K::ESZ;
+        if (K::VF == GC_C64) {
+            for (int x = lane; x < L; x += 32)
+                reinterpret_cast<float2 *>(dst)[x] =
+                    ok ? reinterpret_cast<const float2 *>(src)[x] : make_float2(0.f, 0.f);
+        } else if (K::VF == GC_C32H) {
+            for (int x = lane; x < L; x += 32)
+                reinterpret_cast<unsigned int *>(dst)[x] = ok ? reinterpret_cast<const unsigned int *>(src)[x] : 0u;
+        } else {
+            // four bytes at a time from two aligned words; what comes along
+            // past the row meets zero coefficients
+            const int a = (int)(src - raw), sh = 8 * (a & 3);
+            const unsigned int *w = reinterpret_cast<const unsigned int *>(raw) + (a >> 2);
+            for (int x = lane; 4 * x < L; x += 32)
+                reinterpret_cast<unsigned int *>(dst)[x] = ok ? __funnelshift_r(w[x], w[x + 1], sh) : 0u;
+        }
+    }
+}
+
+template <class K, int kMode>
+__global__ void __launch_bounds__(K::NTHREADS, kMode == kStageBulk && K::VF == GC_C32H && K::M == 64 ? 3 : K::MINB)
 fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + K::OFF_BAR);
     float2 *tws = reinterpret_cast<float2 *>(smem + K::OFF_TW);
     float2 *coef = reinterpret_cast<float2 *>(smem + K::OFF_COEF);
     unsigned char *stage0 = smem + K::OFF_STAGE;
-    float2 *inter = reinterpret_cast<float2 *>(smem + K::OFF_INTER);
+    // this thread's residue of the CTA's, its place among that residue's threads
+    const int qg = K::QG == 1 ? 0 : threadIdx.x / K::GTHREADS, gtid = threadIdx.x - qg * K::GTHREADS;
+    float2 *inter = reinterpret_cast<float2 *>(smem + K::OFF_INTER) + qg * K::INTER;
     __shared__ int s_err;
+    constexpr bool kTMA = kMode == kStageTiled;   // tiled copies
+    constexpr int NST = K::NSTAGE;
 
     const int tid = threadIdx.x;
     const int L = p.L;
@@ -176,10 +226,13 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
         const cf w = c_tw.v[e * (256 / K::M)];
         tws[e] = make_float2(w.x, w.y);
     }
-    for (int i = tid; i < K::GNT * K::LMAX * K::IROW; i += K::NTHREADS) inter[i] = make_float2(0.f, 0.f);
+    for (int i = gtid; i < K::INTER; i += K::GTHREADS) inter[i] = make_float2(0.f, 0.f);
+    if (kMode == kStageBulk)   // columns past L of the padded rows stay zero
+        for (int i = tid; i < K::STAGE_BYTES / 16; i += K::NTHREADS)
+            reinterpret_cast<uint4 *>(stage0)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
         s_err = 0;
-        if (kTMA) {
+        if (kMode != kStagePlain) {
             gc_mbar_init(&bars[0], 1);
             gc_mbar_init(&bars[1], 1);
             gc_fence_mbar_init();
@@ -188,8 +241,8 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
     __syncthreads();
 
     // column item owned by this thread (fixed for the whole kernel)
-    const int g = tid / K::NCOL;
-    const int col = tid % K::NCOL;
+    const int g = gtid / K::NCOL;
+    const int col = gtid % K::NCOL;
     const int kxl = col % K::MX;
     const int s2 = col / K::MX;
     const int n_it = p.chunk_len / K::GNT;
@@ -197,9 +250,10 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
     uint32_t ld_count = 0, use_count = 0;   // TMA loads issued / consumed (phase tracking)
 
     for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
-        const int q = item % K::R;
-        const int chunk = (item / K::R) % p.n_chunks;
-        const int c = item / (K::R * p.n_chunks);
+        constexpr int RQ = K::R / K::QG;
+        const int q = (item % RQ) * K::QG + qg;
+        const int chunk = (item / RQ) % p.n_chunks;
+        const int c = item / (RQ * p.n_chunks);
         const int t0 = chunk * p.chunk_len;
 
         // calibration coefficients 1/g_i = conj(g)/|g|^2 in the padded layout
@@ -222,13 +276,35 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
             coef[i] = cc;
         }
         if (kTMA && tid == 0) {
-            for (int k = 0; k < 2 && k < n_it; ++k) {
-                unsigned char *dst = stage0 + (ld_count & 1u) * kStageStride;
-                gc_mbar_expect_tx(&bars[ld_count & 1u], K::STAGE_BYTES);
-                gc_tma_load_4d(dst, &tmap, &bars[ld_count & 1u], 0, 0, t0 + k * K::GNT, c);
+            for (int k = 0; k < NST && k < n_it; ++k) {
+                unsigned char *dst = stage0 + (ld_count % NST) * kStageStride;
+                gc_mbar_expect_tx(&bars[ld_count % NST], K::STAGE_BYTES);
+                gc_tma_load_4d(dst, &tmap, &bars[ld_count % NST], 0, 0, t0 + k * K::GNT, c);
                 ++ld_count;
             }
         }
+        // bulk copies: whole 16-byte units around the samples at t; the last
+        // samples of the buffer, whose units would reach past its end, and
+        // samples past T are left to plain loads
+        unsigned char *raw = NST > 1 ? stage0 + kStageStride : smem + K::SMEM;
+        const size_t sample = (size_t)L * L * K::ESZ;
+        auto span = [&](int t, size_t &lo, uint32_t &bytes) -> bool {
+            const size_t s0 = ((size_t)c * p.T + t) * sample, s1 = s0 + (size_t)min(K::GNT, p.T - t) * sample;
+            lo = s0 & ~(size_t)15;
+            const size_t hi = (s1 + 15) & ~(size_t)15;
+            bytes = (uint32_t)(hi - lo);
+            return t < p.T && hi <= (size_t)p.C * p.T * sample;
+        };
+        auto bulk_issue = [&](int t) {
+            size_t lo;
+            uint32_t bytes;
+            if (!span(t, lo, bytes)) return;
+            gc_fence_proxy_async();
+            gc_mbar_expect_tx(&bars[0], bytes);
+            gc_bulk_load(raw, static_cast<const unsigned char *>(p.volt) + lo, bytes, &bars[0]);
+            ++ld_count;
+        };
+        if (kMode == kStageBulk && tid == 0) bulk_issue(t0);
         __syncthreads();
 
         float acc[K::F2];
@@ -239,9 +315,9 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
             const int t = t0 + it * K::GNT;
             unsigned char *stage;
             if (kTMA) {
-                const uint32_t buf = use_count & 1u;
+                const uint32_t buf = use_count % NST;
                 stage = stage0 + buf * kStageStride;
-                if (!gc_mbar_wait(&bars[buf], (use_count >> 1) & 1u, GC_WAIT_LIMIT_NS)) {
+                if (!gc_mbar_wait(&bars[buf], (use_count / NST) & 1u, GC_WAIT_LIMIT_NS)) {
                     atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
                     s_err = 1;
                 } else {
@@ -249,6 +325,25 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
                 }
                 __syncthreads();
                 if (s_err) break;
+            } else if (kMode == kStageBulk) {
+                stage = stage0;
+                size_t lo;
+                uint32_t bytes;
+                if (span(t, lo, bytes)) {
+                    if (!gc_mbar_wait(&bars[0], use_count & 1u, GC_WAIT_LIMIT_NS)) {
+                        atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
+                        s_err = 1;
+                    } else {
+                        ++use_count;
+                    }
+                    __syncthreads();
+                    if (s_err) break;
+                    repack_rows<K>(p, stage, raw, (int)(((size_t)c * p.T + t) * sample - lo), t);
+                } else {
+                    stage_plain<K>(p, stage, c, t);
+                }
+                __syncthreads();
+                if (tid == 0 && it + 1 < n_it) bulk_issue(t + K::GNT);
             } else {
                 stage = stage0;
                 stage_plain<K>(p, stage, c, t);
@@ -256,7 +351,7 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
             }
 
             // ---------------- row pass
-            for (int r = tid; r < rows_per_it; r += K::NTHREADS) {
+            for (int r = gtid; r < rows_per_it; r += K::GTHREADS) {
                 const int y = r % L;
                 const int rest = r / L;
                 const int u = rest % K::GNT;
@@ -328,12 +423,12 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
             }
             __syncthreads();
 
-            // refill the consumed stage with the samples two iterations ahead
-            if (kTMA && tid == 0 && it + 2 < n_it) {
+            // refill the consumed stage with the samples NSTAGE iterations ahead
+            if (kTMA && tid == 0 && it + NST < n_it) {
                 gc_fence_proxy_async();
-                unsigned char *dst = stage0 + (ld_count & 1u) * kStageStride;
-                gc_mbar_expect_tx(&bars[ld_count & 1u], K::STAGE_BYTES);
-                gc_tma_load_4d(dst, &tmap, &bars[ld_count & 1u], 0, 0, t + 2 * K::GNT, c);
+                unsigned char *dst = stage0 + (ld_count % NST) * kStageStride;
+                gc_mbar_expect_tx(&bars[ld_count % NST], K::STAGE_BYTES);
+                gc_tma_load_4d(dst, &tmap, &bars[ld_count % NST], 0, 0, t + NST * K::GNT, c);
                 ++ld_count;
             }
 
@@ -394,10 +489,11 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
         }
     }
 
-    if (kTMA && s_err && tid == 0) {
+    if (kMode != kStagePlain && s_err && tid == 0) {
         // let copies still in flight land before the CTA exits (bounded)
+        constexpr uint32_t nb = kTMA ? NST : 1;
         while (use_count < ld_count) {
-            gc_mbar_wait(&bars[use_count & 1u], (use_count >> 1) & 1u, GC_WAIT_LIMIT_NS / 10);
+            gc_mbar_wait(&bars[use_count % nb], (use_count / nb) & 1u, GC_WAIT_LIMIT_NS / 10);
             ++use_count;
         }
     }
@@ -533,6 +629,49 @@ fftcorr_finalize_cols(const float2 *__restrict__ Q, float2 *__restrict__ vunique
 }
 
 // ----------------------------------------------------------------- host side
+// Staging of a call: tiled copies where the rows allow them, else bulk copies
+// where the buffer is 16-byte aligned (and, with a single stage, their space
+// fits behind the CTA's); `smem`: the dynamic shared memory.
+template <class K>
+int stage_mode(const void *volt, int L, bool tiled, size_t &smem) {
+    smem = K::SMEM;
+    if (!gc_aligned(volt, 16)) return kStagePlain;
+    if (tiled && ((size_t)L * K::ESZ) % 16 == 0) return kStageTiled;
+    if (K::M < 64) return kStagePlain;   // rows too short for a warp each (L = 13: plain 106, bulk 137 us)
+    if (K::NSTAGE > 1) return L < K::LMAX ? kStageBulk : kStagePlain;
+    const size_t more = K::SMEM + ((size_t)K::GNT * L * L * K::ESZ + 63) / 16 * 16;
+    if (more > 227u * 1024u - 256u) return kStagePlain;
+    smem = more;
+    return kStageBulk;
+}
+using AccKernel = void (*)(const CUtensorMap, const Params);
+template <class K>
+AccKernel acc_kernel(int mode) {
+    return mode == kStageTiled ? fftcorr_accumulate<K, kStageTiled>
+                               : (mode == kStageBulk ? fftcorr_accumulate<K, kStageBulk> : fftcorr_accumulate<K, kStagePlain>);
+}
+
+// CTAs to launch for `items` equal items: k per SM, 1 <= k <= occ, for the
+// least time, k resident CTAs taking about k^a times as long for one item each
+// and the last wave as many as it has -- so a full last wave of fewer can beat
+// a nearly empty one.  Measured: a = 0.75 (two against one 1.55 to 1.67, three
+// against two 1.41), 0.35 for binary16 at M = 64 from bulk copies (1.13).
+int launch_ctas(long items, int occ, int sms, double a) {
+    int best = 1;
+    double least = 0.0;
+    for (int k = 1; k <= occ; ++k) {
+        const long full = items / ((long)k * sms), left = items - full * k * sms;
+        const double t = full * pow((double)k, a) + pow((double)((left + sms - 1) / sms), a);
+        if (k == 1 || t < least - 1e-9) {
+            least = t;
+            best = k;
+        }
+    }
+    return (int)std::min<long>(items, (long)best * sms);
+}
+template <class K>
+constexpr double kCtaCost = K::VF == GC_C32H && K::M == 64 ? 0.35 : 0.75;
+
 template <class K>
 CUtensorMapDataType tma_dtype() {
     return K::VF == GC_C64 ? CU_TENSOR_MAP_DATA_TYPE_UINT64
@@ -546,14 +685,17 @@ struct Launcher {
     static gc_status run(gc_ctx *ctx, const void *volt, int L, int C, int T, const float *gains,
                          float *vunique, cudaStream_t stream, const unsigned char *h_mask = nullptr) {
         const int N = L * L;
-        const bool tma = gc_aligned(volt, 16) && ((size_t)L * K::ESZ) % 16 == 0;
-        auto kern = tma ? fftcorr_accumulate<K, true> : fftcorr_accumulate<K, false>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM);
+        size_t smem;
+        const int mode = stage_mode<K>(volt, L, true, smem);
+        const bool tma = mode == kStageTiled;
+        const AccKernel kern = acc_kernel<K>(mode);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(fftcorr_accumulate)");
         int occ = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, K::NTHREADS, K::SMEM);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, K::NTHREADS, smem);
         if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(fftcorr_accumulate)");
         const int slots = occ * ctx->sm_count;
+        const int wave = K::CHUNK_CTAS > 0 ? K::CHUNK_CTAS * ctx->sm_count : slots;
 
         // time chunking: chunks of <= 512 samples, chosen so the work items
         // fill whole waves of the resident CTAs
@@ -565,8 +707,8 @@ struct Launcher {
             const int len = ((T + n - 1) / n + step - 1) / step * step;
             const int nn = (T + len - 1) / len;
             const long items = (long)C * K::R * nn;
-            const long waves = (items + slots - 1) / slots;
-            const double eff = (double)C * K::R * T / ((double)waves * slots * len);
+            const long waves = (items + wave - 1) / wave;
+            const double eff = (double)C * K::R * T / ((double)waves * wave * len);
             if (eff > best_eff + 1e-9) {
                 best_eff = eff;
                 best_n = nn;
@@ -586,7 +728,7 @@ struct Launcher {
         p.T = T;
         p.chunk_len = best_len;
         p.n_chunks = best_n;
-        p.n_items = C * K::R * best_n;
+        p.n_items = C * (K::R / K::QG) * best_n;
         const size_t part_bytes = ((size_t)C * best_n * K::M * K::M * sizeof(float) + 255) / 256 * 256;
         const size_t q_bytes = K::M > 128 ? (size_t)C * K::M * (2 * L - 1) * sizeof(float2) : 0;
         const int Wd = 2 * L - 1;
@@ -627,9 +769,10 @@ struct Launcher {
             st = gc_encode_tiled(ctx, &tmap, tma_dtype<K>(), 4, const_cast<void *>(volt), dims, strides, box);
             if (st != GC_OK) return st;
         }
-        const int grid = (int)std::min<long>(p.n_items, slots);
+        const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, ctx->sm_count, kCtaCost<K>)
+                                           : (int)std::min<long>(p.n_items, slots);
         int rec = gc_prof_begin(ctx, stream, "fftcorr_accumulate");
-        kern<<<grid, K::NTHREADS, K::SMEM, stream>>>(tmap, p);
+        kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
         gc_prof_end(ctx, stream, rec);
         e = cudaGetLastError();
         if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "launch fftcorr_accumulate");
@@ -658,11 +801,18 @@ struct Launcher {
     }
 };
 
-// configurations per FFT side (see the design notes for the smem budget)
+// configurations per FFT side.  The 64-point complex64 one lets three CTAs live
+// on an SM (168 registers, one stage) instead of two, the 128-point complex64 and
+// binary16 ones two instead of one (one stage): 256 channels of 32x32
+// complex64, 4096 samples, 5.72 -> 5.54 ms; 32 of 48x48, 500 samples, 1.39 ->
+// 1.08 ms; 32 of 64x64 binary16, 500 samples, 1.78 -> 1.49 ms.  The 64-point
+// binary16 one does so from bulk copies only (331 antennas 2.16 -> 1.91 ms;
+// from tiled copies 618 -> 640 us).  4+4-bit voltages at M = 64 spill at three
+// CTAs and were slower (811 -> 888 us).
 using CfgC16 = Cfg<16, 1, 16, 16, 2, 8, GC_C64>;
 using CfgC32 = Cfg<32, 1, 32, 32, 2, 4, GC_C64>;
-using CfgC64 = Cfg<64, 1, 32, 32, 2, 1, GC_C64>;
-using CfgC128 = Cfg<128, 4, 32, 32, 1, 1, GC_C64>;
+using CfgC64 = Cfg<64, 1, 32, 32, 2, 1, GC_C64, 3, 1, 1, 2>;
+using CfgC128 = Cfg<128, 4, 32, 32, 1, 1, GC_C64, 2, 1, 1, 1>;
 using CfgI16 = Cfg<16, 1, 16, 16, 2, 8, GC_I4C>;
 using CfgI32 = Cfg<32, 1, 32, 32, 2, 4, GC_I4C>;
 using CfgI64 = Cfg<64, 1, 32, 32, 2, 1, GC_I4C>;
@@ -674,13 +824,16 @@ using CfgI128b = Cfg<128, 4, 32, 32, 2, 1, GC_I4C, 2>;
 using CfgC64b = Cfg<64, 1, 32, 32, 1, 2, GC_C64>;
 // M = 256 (L = 65..128): 4+4-bit only -- one complex64 or binary16 grid sample
 // (128 rows of 1 KB / 512 B) does not fit a double-buffered stage beside the
-// 133 KB coefficient table.  Eight k_x residues, one sample per iteration,
-// one CTA of 256 threads per SM (201 KB shared memory).
-using CfgI256 = Cfg<256, 8, 16, 32, 1, 1, GC_I4C>;
+// 133 KB coefficient table.  Eight k_x residues, two of them side by side in a
+// CTA of 512 threads that share the samples and the coefficients (222 KB
+// shared memory with one stage, refilled during the column pass).  48 channels
+// of 128x128 antennas, 1100 samples: 16.1 ms, 19.3 ms with one residue and
+// 256 threads an SM and two stages.
+using CfgI256 = Cfg<256, 8, 16, 32, 1, 1, GC_I4C, 1, 1, 2>;
 using CfgH16 = Cfg<16, 1, 16, 16, 2, 8, GC_C32H>;
 using CfgH32 = Cfg<32, 1, 32, 32, 2, 4, GC_C32H>;
-using CfgH64 = Cfg<64, 1, 32, 32, 2, 1, GC_C32H>;
-using CfgH128 = Cfg<128, 4, 32, 32, 1, 2, GC_C32H>;
+using CfgH64 = Cfg<64, 1, 32, 32, 2, 1, GC_C32H, 1, 2, 1, 2>;
+using CfgH128 = Cfg<128, 4, 32, 32, 1, 2, GC_C32H, 2, 1, 1, 1>;
 
 // Row stage on the tensor cores (gc_fftcorr_tc.cu), then the same finalize.
 gc_status tc_correlate(gc_ctx *ctx, const void *volt, int L, int C, int T, const float *gains, float *vunique,
@@ -822,16 +975,18 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
     const int n_min = std::max(1, (T + 511) / 512);      // chunks of <= 512 samples
     if (per_chunk * n_min > kNoallocScratchBytes) return GC_EINVAL;
     const int n_cap = (int)std::min<size_t>(kNoallocScratchBytes / per_chunk, (size_t)n_min + 64);
-    bool tma = gc_aligned(volt, 16) && ((size_t)L * K::ESZ) % 16 == 0 && g_noalloc_encode != nullptr;
-    auto kern = tma ? fftcorr_accumulate<K, true> : fftcorr_accumulate<K, false>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, K::SMEM) != cudaSuccess)
+    size_t smem;
+    const int mode = stage_mode<K>(volt, L, g_noalloc_encode != nullptr, smem);
+    const bool tma = mode == kStageTiled;
+    const AccKernel kern = acc_kernel<K>(mode);
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return GC_ECUDA;
     int occ = 0, sms = 0, dev = 0;
     cudaGetDevice(&dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, K::NTHREADS, K::SMEM) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, K::NTHREADS, smem) != cudaSuccess ||
         occ < 1 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return GC_ECUDA;
-    const int slots = occ * sms;
+    const int slots = occ * sms, wave = K::CHUNK_CTAS > 0 ? K::CHUNK_CTAS * sms : slots;
     const int step = K::GNT;
     int best_n = n_min, best_len = ((T + n_min - 1) / n_min + step - 1) / step * step;
     double best_eff = -1.0;
@@ -840,8 +995,8 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
         const int nn = (T + len - 1) / len;
         if (nn > n_cap) continue;
         const long items = (long)C * K::R * nn;
-        const long waves = (items + slots - 1) / slots;
-        const double eff = (double)C * K::R * T / ((double)waves * slots * len);
+        const long waves = (items + wave - 1) / wave;
+        const double eff = (double)C * K::R * T / ((double)waves * wave * len);
         if (eff > best_eff + 1e-9) {
             best_eff = eff;
             best_n = nn;
@@ -858,7 +1013,7 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
     p.T = T;
     p.chunk_len = best_len;
     p.n_chunks = best_n;
-    p.n_items = C * K::R * best_n;
+    p.n_items = C * (K::R / K::QG) * best_n;
 
     CUtensorMap tmap;
     memset(&tmap, 0, sizeof tmap);
@@ -878,8 +1033,8 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return GC_ECUDA;
     }
-    const int grid = (int)std::min<long>(p.n_items, slots);
-    kern<<<grid, K::NTHREADS, K::SMEM, stream>>>(tmap, p);
+    const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, sms, kCtaCost<K>) : (int)std::min<long>(p.n_items, slots);
+    kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
     if (cudaGetLastError() != cudaSuccess) return GC_ECUDA;
     const int W = 2 * L - 1;
     const size_t fsmem = (size_t)K::M * K::M * 4 + (size_t)K::M * W * 8 + K::M * 8;
