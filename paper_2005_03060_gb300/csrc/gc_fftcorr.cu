@@ -500,19 +500,41 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
 }
 
 // ----------------------------------------------------------------- finalize
+// What bounds it: the twiddle gathers from shared memory (lanes take
+// neighbouring lags), so a thread keeps kFinTile outputs that share them, and
+// the FP64 divisions by T N_d (a table over the products of two sides, not one
+// division per lag).  256 channels of the 64x64 grid: 600 us, 1100 us with one
+// output a thread at a time and 256 threads; 48 of 128x128 by the two-pass form
+// below: 970 against 1115 us.  FFTs of M < 64 have too few outputs for that (200
+// channels at M = 16: 113 us with one a thread, 118 us with four) and keep
+// one.  The sum of each output runs in the same order in all forms.
+constexpr int kFinTile = 4;
+constexpr int fin_tile(int M) { return M >= 64 ? kFinTile : 1; }
+constexpr int fin_threads(int M) { return M >= 64 ? 1024 : 256; }
+__host__ __device__ constexpr size_t fin_smem(int M, int L) {
+    return (size_t)M * M * 4 + (size_t)M * (2 * L - 1) * 8 + (size_t)M * 8 + (size_t)L * L * 4;
+}
+
 template <int M>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(fin_threads(M))
 fftcorr_finalize(const float *__restrict__ ppart, int n_parts, float2 *__restrict__ vunique, int L, int T,
                  const float *__restrict__ ndtab, unsigned int *status) {
+    constexpr int kTile = fin_tile(M);
     extern __shared__ __align__(128) unsigned char smem[];
     float *P = reinterpret_cast<float *>(smem);                 // [M][M]
     float2 *Q = reinterpret_cast<float2 *>(smem + M * M * 4);   // [M][W]
     float2 *tws = Q + M * (2 * L - 1);                          // [M]
+    float *norm = reinterpret_cast<float *>(tws + M);           // [L][L]: 1 / (M^2 T N_d), N_d = (i + 1)(j + 1)
     const int c = blockIdx.x, W = 2 * L - 1;
     for (int e = threadIdx.x; e < M; e += blockDim.x) {
         const cf w = c_tw.v[e * (256 / M)];
         tws[e] = make_float2(w.x, w.y);
     }
+    if (!ndtab)
+        for (int e = threadIdx.x; e < L * L; e += blockDim.x) {
+            const int i = e / L, j = e - i * L;
+            if (j >= i) norm[e] = norm[j * L + i] = (float)(1.0 / ((double)M * M * (double)T * (double)((i + 1) * (j + 1))));
+        }
     const float *src = ppart + (size_t)c * n_parts * M * M;
     for (int k = threadIdx.x; k < M * M; k += blockDim.x) {
         double s = 0.0;
@@ -522,34 +544,69 @@ fftcorr_finalize(const float *__restrict__ ppart, int n_parts, float2 *__restric
     }
     __syncthreads();
     // Q[ky][dx] = sum_kx P[ky][kx] exp(+2 pi i kx dx / M)
-    for (int idx = threadIdx.x; idx < M * W; idx += blockDim.x) {
-        const int ky = idx / W, dx = idx % W - (L - 1);
-        float re = 0.f, im = 0.f;
-        for (int kx = 0; kx < M; ++kx) {
-            const float2 w = tws[(kx * dx) & (M - 1)];   // conj gives the + sign
-            const float pv = P[ky * M + kx];
-            re = fmaf(pv, w.x, re);
-            im = fmaf(-pv, w.y, im);
+    for (int idx = threadIdx.x; idx < M / kTile * W; idx += blockDim.x) {
+        const int kg = idx / W, dx = idx - kg * W - (L - 1);
+        const float *pk = P + kTile * kg * M;
+        float re[kTile], im[kTile];
+#pragma unroll
+        for (int u = 0; u < kTile; ++u) re[u] = im[u] = 0.f;
+        int e = 0;   // kx dx mod M
+#pragma unroll 2
+        for (int kx = 0; kx < M; kx += 4) {
+            float4 pv[kTile];
+#pragma unroll
+            for (int u = 0; u < kTile; ++u) pv[u] = *reinterpret_cast<const float4 *>(pk + u * M + kx);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float2 w = tws[e];   // conj gives the + sign
+                e = (e + dx) & (M - 1);
+#pragma unroll
+                for (int u = 0; u < kTile; ++u) {
+                    const float q = v == 0 ? pv[u].x : (v == 1 ? pv[u].y : (v == 2 ? pv[u].z : pv[u].w));
+                    re[u] = fmaf(q, w.x, re[u]);
+                    im[u] = fmaf(-q, w.y, im[u]);
+                }
+            }
         }
-        Q[ky * W + (dx + L - 1)] = make_float2(re, im);
+#pragma unroll
+        for (int u = 0; u < kTile; ++u) Q[(kTile * kg + u) * W + dx + L - 1] = make_float2(re[u], im[u]);
     }
     __syncthreads();
     // R[dy][dx] = (1/M^2) sum_ky Q[ky][dx] exp(+2 pi i ky dy / M); V = R / (T N_d)
-    for (int idx = threadIdx.x; idx < W * W; idx += blockDim.x) {
-        const int dyi = idx / W, dxi = idx % W;
-        const int dy = dyi - (L - 1), dx = dxi - (L - 1);
-        float re = 0.f, im = 0.f;
-        for (int ky = 0; ky < M; ++ky) {
-            const float2 w = tws[(ky * dy) & (M - 1)];
-            const float2 qv = Q[ky * W + dxi];
-            // qv * conj(w)
-            re = fmaf(qv.x, w.x, fmaf(qv.y, w.y, re));
-            im = fmaf(qv.y, w.x, fmaf(-qv.x, w.y, im));
+    for (int idx = threadIdx.x; idx < (W + kTile - 1) / kTile * W; idx += blockDim.x) {
+        const int dg = idx / W, dxi = idx - dg * W, dx = dxi - (L - 1), dy0 = kTile * dg - (L - 1);
+        float re[kTile], im[kTile];
+        int e[kTile];
+#pragma unroll
+        for (int u = 0; u < kTile; ++u) {
+            re[u] = im[u] = 0.f;
+            e[u] = 0;
         }
-        // N_d: pairs per lag (a partly occupied lattice passes its table)
-        const double nd = ndtab ? (double)ndtab[idx] : (double)((L - (dx < 0 ? -dx : dx)) * (L - (dy < 0 ? -dy : dy)));
-        const float s = nd > 0.0 ? (float)(1.0 / ((double)M * M * (double)T * nd)) : 0.f;
-        vunique[(size_t)c * W * W + idx] = make_float2(re * s, im * s);
+#pragma unroll 4
+        for (int ky = 0; ky < M; ++ky) {
+            const float2 qv = Q[ky * W + dxi];
+#pragma unroll
+            for (int u = 0; u < kTile; ++u) {
+                const float2 w = tws[e[u]];
+                e[u] = (e[u] + dy0 + u) & (M - 1);
+                // qv * conj(w)
+                re[u] = fmaf(qv.x, w.x, fmaf(qv.y, w.y, re[u]));
+                im[u] = fmaf(qv.y, w.x, fmaf(-qv.x, w.y, im[u]));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kTile; ++u) {
+            const int dy = dy0 + u, o = (dy + L - 1) * W + dxi;
+            if (dy >= L) continue;
+            float s;
+            if (ndtab) {   // pairs per lag of a partly occupied lattice
+                const double nd = (double)ndtab[o];
+                s = nd > 0.0 ? (float)(1.0 / ((double)M * M * (double)T * nd)) : 0.f;
+            } else {
+                s = norm[(L - 1 - abs(dx)) * L + L - 1 - abs(dy)];
+            }
+            vunique[(size_t)c * W * W + o] = make_float2(re[u] * s, im[u] * s);
+        }
     }
 }
 
@@ -581,16 +638,25 @@ fftcorr_finalize_rows(const float *__restrict__ ppart, int n_parts, float2 *__re
         P[k / M][k % M] = (float)s;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < kFinRows * W; idx += blockDim.x) {
-        const int r = idx / W, dx = idx % W - (L - 1);
-        float re = 0.f, im = 0.f;
+    // a thread takes all rows of a lag: they share its twiddles
+    for (int i = threadIdx.x; i < W; i += blockDim.x) {
+        const int dx = i - (L - 1);
+        float re[kFinRows], im[kFinRows];
+#pragma unroll
+        for (int r = 0; r < kFinRows; ++r) re[r] = im[r] = 0.f;
+        int e = 0;   // kx dx mod M
         for (int kx = 0; kx < M; ++kx) {
-            const float2 w = tws[(kx * dx) & (M - 1)];
-            const float pv = P[r][kx];
-            re = fmaf(pv, w.x, re);
-            im = fmaf(-pv, w.y, im);
+            const float2 w = tws[e];
+            e = (e + dx) & (M - 1);
+#pragma unroll
+            for (int r = 0; r < kFinRows; ++r) {
+                const float pv = P[r][kx];
+                re[r] = fmaf(pv, w.x, re[r]);
+                im[r] = fmaf(-pv, w.y, im[r]);
+            }
         }
-        Q[((size_t)c * M + ky0 + r) * W + (dx + L - 1)] = make_float2(re, im);
+#pragma unroll
+        for (int r = 0; r < kFinRows; ++r) Q[((size_t)c * M + ky0 + r) * W + i] = make_float2(re[r], im[r]);
     }
 }
 
@@ -611,20 +677,38 @@ fftcorr_finalize_cols(const float2 *__restrict__ Q, float2 *__restrict__ vunique
         Qs[ky][j] = j < ncol ? Q[((size_t)c * M + ky) * W + dx0 + j] : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < W * ncol; idx += blockDim.x) {
-        const int dyi = idx / ncol, j = idx % ncol;
-        const int dy = dyi - (L - 1), dxi = dx0 + j, dx = dxi - (L - 1);
-        float re = 0.f, im = 0.f;
-        for (int ky = 0; ky < M; ++ky) {
-            const float2 w = tws[(ky * dy) & (M - 1)];
-            const float2 qv = Qs[ky][j];
-            re = fmaf(qv.x, w.x, fmaf(qv.y, w.y, re));
-            im = fmaf(qv.y, w.x, fmaf(-qv.x, w.y, im));
+    // a thread takes kFinTile lags of a column: they share its values of Q
+    for (int idx = threadIdx.x; idx < (W + kFinTile - 1) / kFinTile * kFinCols; idx += blockDim.x) {
+        const int dg = idx / kFinCols, j = idx % kFinCols, dxi = dx0 + j, dx = dxi - (L - 1);
+        if (j >= ncol) continue;
+        const int dy0 = kFinTile * dg - (L - 1);
+        float re[kFinTile], im[kFinTile];
+        int e[kFinTile];
+#pragma unroll
+        for (int u = 0; u < kFinTile; ++u) {
+            re[u] = im[u] = 0.f;
+            e[u] = 0;
         }
-        const double nd = ndtab ? (double)ndtab[(size_t)dyi * W + dxi]
-                                : (double)((L - (dx < 0 ? -dx : dx)) * (L - (dy < 0 ? -dy : dy)));
-        const float s = nd > 0.0 ? (float)(1.0 / ((double)M * M * (double)T * nd)) : 0.f;
-        vunique[(size_t)c * W * W + (size_t)dyi * W + dxi] = make_float2(re * s, im * s);
+#pragma unroll 4
+        for (int ky = 0; ky < M; ++ky) {
+            const float2 qv = Qs[ky][j];
+#pragma unroll
+            for (int u = 0; u < kFinTile; ++u) {
+                const float2 w = tws[e[u]];
+                e[u] = (e[u] + dy0 + u) & (M - 1);
+                re[u] = fmaf(qv.x, w.x, fmaf(qv.y, w.y, re[u]));
+                im[u] = fmaf(qv.y, w.x, fmaf(-qv.x, w.y, im[u]));
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kFinTile; ++u) {
+            const int dy = dy0 + u;
+            if (dy >= L) continue;
+            const size_t o = (size_t)(dy + L - 1) * W + dxi;
+            const double nd = ndtab ? (double)ndtab[o] : (double)((L - abs(dx)) * (L - abs(dy)));
+            const float s = nd > 0.0 ? (float)(1.0 / ((double)M * M * (double)T * nd)) : 0.f;
+            vunique[(size_t)c * W * W + o] = make_float2(re[u] * s, im[u] * s);
+        }
     }
 }
 
@@ -787,12 +871,12 @@ struct Launcher {
                 Q, reinterpret_cast<float2 *>(vunique), L, T, ndtab);
             gc_prof_end(ctx, stream, rec);
         } else {
-            const size_t fsmem = (size_t)K::M * K::M * 4 + (size_t)K::M * W * 8 + K::M * 8;
+            const size_t fsmem = fin_smem(K::M, L);
             auto fin = fftcorr_finalize<K::M>;
             e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
             if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(fftcorr_finalize)");
             rec = gc_prof_begin(ctx, stream, "fftcorr_finalize");
-            fin<<<C, 256, fsmem, stream>>>(p.ppart, best_n, reinterpret_cast<float2 *>(vunique), L, T, ndtab, p.status);
+            fin<<<C, fin_threads(K::M), fsmem, stream>>>(p.ppart, best_n, reinterpret_cast<float2 *>(vunique), L, T, ndtab, p.status);
             gc_prof_end(ctx, stream, rec);
         }
         e = cudaGetLastError();
@@ -842,13 +926,12 @@ gc_status tc_correlate(gc_ctx *ctx, const void *volt, int L, int C, int T, const
     int n_chunks = 0;
     gc_status st = gc_fft_tc_run(ctx, volt, L, C, T, gains, &ppart, &n_chunks, stream);
     if (st != GC_OK) return st;
-    const int W = 2 * L - 1;
-    const size_t fsmem = (size_t)128 * 128 * 4 + (size_t)128 * W * 8 + 128 * 8;
+    const size_t fsmem = fin_smem(128, L);
     auto fin = fftcorr_finalize<128>;
     cudaError_t e = cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
     if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(fftcorr_finalize)");
     const int rec = gc_prof_begin(ctx, stream, "fftcorr_finalize");
-    fin<<<C, 256, fsmem, stream>>>(ppart, n_chunks, reinterpret_cast<float2 *>(vunique), L, T, nullptr,
+    fin<<<C, fin_threads(128), fsmem, stream>>>(ppart, n_chunks, reinterpret_cast<float2 *>(vunique), L, T, nullptr,
                                    ctx->status_dev);
     gc_prof_end(ctx, stream, rec);
     e = cudaGetLastError();
@@ -1036,12 +1119,11 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
     const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, sms, kCtaCost<K>) : (int)std::min<long>(p.n_items, slots);
     kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
     if (cudaGetLastError() != cudaSuccess) return GC_ECUDA;
-    const int W = 2 * L - 1;
-    const size_t fsmem = (size_t)K::M * K::M * 4 + (size_t)K::M * W * 8 + K::M * 8;
+    const size_t fsmem = fin_smem(K::M, L);
     auto fin = fftcorr_finalize<K::M>;
     if (cudaFuncSetAttribute(fin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem) != cudaSuccess)
         return GC_ECUDA;
-    fin<<<C, 256, fsmem, stream>>>(p.ppart, best_n, reinterpret_cast<float2 *>(vunique), L, T, nullptr,
+    fin<<<C, fin_threads(K::M), fsmem, stream>>>(p.ppart, best_n, reinterpret_cast<float2 *>(vunique), L, T, nullptr,
                                    p.status);
     if (cudaGetLastError() != cudaSuccess) return GC_ECUDA;
     return GC_OK;
