@@ -23,8 +23,7 @@ namespace {
 
 constexpr int kCThreads = 512;
 constexpr int kCgThreads = 512;   // matrix-free kernels, pair-scatter operator
-constexpr int kCgStThreads = 256; // matrix-free kernels, stencil operator (128 registers a thread), two CTAs per SM
-constexpr int kCgStMost = 512;    // the same, one CTA per SM
+constexpr int kCgStThreads = 256; // matrix-free kernels, stencil operator (128 registers a thread)
 constexpr int kStencilTypes = 16; // baseline-types the stencil operator holds in registers
 // shared arena cap: two CTAs per SM.  Arrays whose hot vectors need more keep
 // them in global memory (L2) at two CTAs per SM -- measured faster than one
@@ -157,20 +156,12 @@ __host__ __device__ inline size_t cg_sten_floats(int N, int n_ubl) {
     const size_t ne = (size_t)N + n_ubl;
     return 2 * ne + 2 * ne + (ne + 1) / 2 + 64;   // q, G, D, coarse index (16 bit)
 }
-// Its other vectors (state, operator output, x, r, z), in shared memory in the
-// wide kernel where there is room beside those and the coarse operators: a CG
-// step reads and writes each of them between barriers (16 channels of 48x48:
-// 1871 us, 2008 us with them in global memory; with two CTAs per SM it gave
-// nothing, 64 channels of 16x16: 674 against 668 us).
-__host__ __device__ inline size_t cg_vec_floats(int N, int n_ubl) {
-    return 5 * (((size_t)2 * (N + n_ubl) + 3) / 4 * 4);
-}
 
 // hot_mode 2: hot vectors and dg in shared memory; 1: hot vectors in shared
 // memory, dg in global; 0: everything in global (L2-resident) memory;
 // 3 (stencil operator): xg, xv and pp in shared memory, the rest in global.
 __device__ CgWork cg_layout(const CalParams &p, char *base, float *smem_arena, int smem_floats, int hot_mode,
-                            bool use_coarse_smem, bool use_vec_smem) {
+                            bool use_coarse_smem) {
     CgWork w;
     w.n = 2 * p.N;
     w.m = 2 * p.n_ubl;
@@ -215,17 +206,6 @@ __device__ CgWork cg_layout(const CalParams &p, char *base, float *smem_arena, i
     if (use_coarse_smem) {
         w.Ca = hot_end;
         w.Cp = hot_end + (size_t)w.nc * w.nc;
-        if (use_vec_smem) {
-            const size_t n4 = (nm + 3) / 4 * 4;
-            // (cg_modes leaves room for rounding the offset up to 16 bytes)
-            float *v = smem_arena + (size_t)(hot_end - smem_arena + 2 * (size_t)w.nc * w.nc + 3) / 4 * 4;
-            w.xg = v;
-            w.xv = v + w.n;
-            w.acc = v + n4;
-            w.x = v + 2 * n4;
-            w.r = v + 3 * n4;
-            w.z = v + 4 * n4;
-        }
     } else {
         w.Ca = takeg((size_t)w.nc * w.nc);
         w.Cp = takeg((size_t)w.nc * w.nc);
@@ -266,12 +246,10 @@ size_t cg_bytes(int N, int n_ubl, int /*P*/) {
 // the issuing warps the way contended shared-memory atomics do.
 // With the stencil operator the arena holds only the gathered vectors (and
 // the coarse operators when they fit beside them).
-size_t cg_arena_bytes(int N, int n_ubl, int L, size_t cap, bool stencil, bool wide = false) {
+size_t cg_arena_bytes(int N, int n_ubl, int L, size_t cap, bool stencil) {
     const size_t h2 = (stencil ? cg_sten_floats(N, n_ubl) : cg_hot_floats(N, n_ubl, true)) * sizeof(float);
     const size_t cf = cg_coarse_floats(L, n_ubl) * sizeof(float);
     const size_t c1 = cf / 2;   // one system: the inversion's shared-memory scratch
-    const size_t vf = cg_vec_floats(N, n_ubl) * sizeof(float) + 16;
-    if (wide && h2 + cf + vf <= cap) return h2 + cf + vf;
     if (h2 + cf <= cap) return h2 + cf;
     if (h2 + c1 <= cap) return h2 + c1;
     if (h2 <= cap) return h2;
@@ -279,16 +257,12 @@ size_t cg_arena_bytes(int N, int n_ubl, int L, size_t cap, bool stencil, bool wi
 }
 
 // the kernel side of the same choice, from the arena size it was given
-template <bool kWide = false>
-__device__ __forceinline__ void cg_modes(const CalParams &p, int smem_floats, int &hot_mode, bool &coarse_smem,
-                                         bool &vec_smem) {
+__device__ __forceinline__ void cg_modes(const CalParams &p, int smem_floats, int &hot_mode, bool &coarse_smem) {
     const size_t cf = cg_coarse_floats(p.L, p.n_ubl), sf = (size_t)smem_floats;
-    vec_smem = false;
     if (p.stencil) {
         const size_t hs = cg_sten_floats(p.N, p.n_ubl);
         hot_mode = hs <= sf ? 3 : 0;
         coarse_smem = hot_mode != 0 && hs + cf <= sf;
-        vec_smem = kWide && coarse_smem && hs + cf + cg_vec_floats(p.N, p.n_ubl) + 4 <= sf;
         return;
     }
     const size_t h2 = cg_hot_floats(p.N, p.n_ubl, true), h1 = cg_hot_floats(p.N, p.n_ubl, false);
@@ -550,10 +524,10 @@ __device__ __forceinline__ float2 rel_obs(const void *vc, int q, float inv) {
     return make_float2((float)v.x * inv, (float)v.y * inv);
 }
 
-template <int VF, int kThreads>
+template <int VF>
 __device__ double rel_resid_pass_t(const CalParams &p, int c, const CgWork &w, bool staged, double *red, float *dmax) {
     constexpr int KT = kStencilTypes;
-    __shared__ float s_tsum[(kThreads / 32) * 3 * KT];
+    __shared__ float s_tsum[(kCgStThreads / 32) * 3 * KT];
     __shared__ int4 s_ra[KT];     // per type: offset d_k, d_y W_k + d_x, b_k, W_k
     __shared__ float4 s_rb[KT];   // per type: 1 / window, V_k
     const int L = p.L, nu = p.n_ubl, N = p.N, bd = blockDim.x;
@@ -659,10 +633,9 @@ __device__ double rel_resid_pass_t(const CalParams &p, int c, const CgWork &w, b
     return rel_resid_finish(p, w, xv, red, dmax, chi, dm);
 }
 
-template <int kThreads>
 __device__ double rel_resid_pass(const CalParams &p, int c, const CgWork &w, bool staged, double *red, float *dmax) {
-    return p.vfmt == GC_C64 ? rel_resid_pass_t<GC_C64, kThreads>(p, c, w, staged, red, dmax)
-                            : rel_resid_pass_t<GC_I4C, kThreads>(p, c, w, staged, red, dmax);
+    return p.vfmt == GC_C64 ? rel_resid_pass_t<GC_C64>(p, c, w, staged, red, dmax)
+                            : rel_resid_pass_t<GC_I4C>(p, c, w, staged, red, dmax);
 }
 
 
@@ -670,10 +643,9 @@ __device__ double rel_resid_pass(const CalParams &p, int c, const CgWork &w, boo
 // q is w.pp, G and q are gathered (shared memory when the arena holds them).
 // Returns this thread's part of q.(A q + mu G q), the CG curvature; acc and
 // the partial sums are complete after the caller's next block reduction.
-template <int kThreads>
 __device__ float rel_op_pass(const CalParams &p, const CgWork &w, float mu) {
     constexpr int KT = kStencilTypes;
-    __shared__ float s_tsum[(kThreads / 32) * 2 * KT];
+    __shared__ float s_tsum[(kCgStThreads / 32) * 2 * KT];
     __shared__ float4 s_ty[KT];   // per type: offset d_k (as int bits), w_k, G_k
     const int L = p.L, nu = p.n_ubl, N = p.N;
     const float2 *q = reinterpret_cast<const float2 *>(w.pp);
@@ -1661,7 +1633,7 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
 // cg_solve_channel; the CG vectors hold (q, w) and the search direction q
 // lives in shared memory beside G, D and the coarse indices.  Convergence
 // tests use the (g, V)-form norms, |r|^2 / G per element.
-template <bool kDense, int kThreads>
+template <bool kDense>
 __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, double cg_tol, int cg_max, double *red,
                                      float *redf) {
     const int ne = p.N + p.n_ubl, L = p.L, nc = w.nc, N = p.N;
@@ -1834,7 +1806,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
         // pass in the instruction stream.)
         float dmax = 0.f;
         const double c2 = kDense ? dense_resid_pass(p, c, w, staged, red, &dmax)
-                                 : rel_resid_pass<kThreads>(p, c, w, staged, red, &dmax);
+                                 : rel_resid_pass(p, c, w, staged, red, &dmax);
         if (staged) {
             staged = false;
             const bool full = c2 <= chi2 * (1.0 + 1e-6) + 1e-30;
@@ -1904,7 +1876,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
             (float)fmin(0.05, fmax(cg_tol, sqrt(sqrt(sqrt((double)bnorm2 / fmax(grad0, 1e-300))))));
         for (int k = 0; k < cg_max && bnorm2 > 0.f; ++k) {
             ++inner;
-            float v1[1] = {kDense ? dense_op_pass(p, w, mu) : rel_op_pass<kThreads>(p, w, mu)};   // acc = A q; q.(A + mu G) q
+            float v1[1] = {kDense ? dense_op_pass(p, w, mu) : rel_op_pass(p, w, mu)};   // acc = A q; q.(A + mu G) q
             fast_sum<1>(v1, sbuf, par);
             if (!(v1[0] > 0.f)) break;
             const float alpha = rz / v1[0];
@@ -2028,21 +2000,19 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
     finish_channel<float>(p, c, w.xg, w.xv, min(it, p.max_iter), st, red, inner);
 }
 
-// kSten: the stencil operator (p.stencil set), launched with up to
-// kCgStThreads threads, or with kWide kCgStMost
-template <bool kPipe, bool kSten, bool kWide>
-__global__ void __launch_bounds__(kSten ? (kWide ? kCgStMost : kCgStThreads) : kCgThreads, kWide ? 1 : 2)
+// kSten: the stencil operator (p.stencil set), launched with kCgStThreads
+template <bool kPipe, bool kSten>
+__global__ void __launch_bounds__(kSten ? kCgStThreads : kCgThreads, 2)
 lincal_cg_kernel(const CalParams p, double cg_tol, int cg_max, int smem_floats) {
     __shared__ double red[32 * 14];
     __shared__ float redf[32 * 14];
     __shared__ float s_rc[2 * kMaxCoarse], s_yc[2 * kMaxCoarse];
     extern __shared__ __align__(16) float arena[];
     int hot_mode;
-    bool coarse_smem, vec_smem;
-    cg_modes<kWide>(p, smem_floats, hot_mode, coarse_smem, vec_smem);
+    bool coarse_smem;
+    cg_modes(p, smem_floats, hot_mode, coarse_smem);
     __shared__ int s_item;
-    CgWork w = cg_layout(p, p.work + (size_t)blockIdx.x * p.work_per_cta, arena, smem_floats, hot_mode, coarse_smem,
-                         vec_smem);
+    CgWork w = cg_layout(p, p.work + (size_t)blockIdx.x * p.work_per_cta, arena, smem_floats, hot_mode, coarse_smem);
     w.rc = s_rc;
     w.yc = s_yc;
     // channels are taken from a device counter: their iteration counts
@@ -2055,7 +2025,7 @@ lincal_cg_kernel(const CalParams p, double cg_tol, int cg_max, int smem_floats) 
         if (c >= p.C) break;
         if constexpr (kSten) {
             if (p.stencil) {
-                cg_solve_channel_rel<false, kWide ? kCgStMost : kCgStThreads>(p, c, w, cg_tol, cg_max, red, redf);
+                cg_solve_channel_rel<false>(p, c, w, cg_tol, cg_max, red, redf);
                 continue;
             }
         }
@@ -2074,7 +2044,7 @@ lincal_cg_dense(const CalParams p, double cg_tol, int cg_max, int smem_floats, i
     __shared__ int s_item;
     const int dn = (int)cg_dense_floats(p.L);
     CgWork w = cg_layout(p, p.work + (size_t)blockIdx.x * p.work_per_cta, arena + dn, smem_floats - dn, 3,
-                         coarse_smem != 0, false);
+                         coarse_smem != 0);
     w.rc = s_rc;
     w.yc = s_yc;
     dense_layout(p, w, arena);
@@ -2086,7 +2056,7 @@ lincal_cg_dense(const CalParams p, double cg_tol, int cg_max, int smem_floats, i
         const int c = s_item;
         __syncthreads();
         if (c >= p.C) break;
-        cg_solve_channel_rel<true, kCgDnThreads>(p, c, w, cg_tol, cg_max, red, redf);
+        cg_solve_channel_rel<true>(p, c, w, cg_tol, cg_max, red, redf);
     }
 }
 
@@ -2126,14 +2096,14 @@ lincal_cg_batched(const __grid_constant__ BatchParams bp) {
         while (slot + 1 < bp.n_arr && bp.prefix[slot + 1] <= item) ++slot;
         const CalParams &p = bp.arr[bp.order[slot]];
         int hot_mode;
-        bool coarse_smem, vec_smem;
-        cg_modes(p, bp.smem_floats, hot_mode, coarse_smem, vec_smem);
-        CgWork w = cg_layout(p, base, arena, bp.smem_floats, hot_mode, coarse_smem, vec_smem);
+        bool coarse_smem;
+        cg_modes(p, bp.smem_floats, hot_mode, coarse_smem);
+        CgWork w = cg_layout(p, base, arena, bp.smem_floats, hot_mode, coarse_smem);
         w.rc = s_rc;
         w.yc = s_yc;
         if constexpr (kSten) {
             if (p.stencil) {
-                cg_solve_channel_rel<false, kCgStThreads>(p, item - bp.prefix[slot], w, bp.cg_tol, bp.cg_max, red, redf);
+                cg_solve_channel_rel<false>(p, item - bp.prefix[slot], w, bp.cg_tol, bp.cg_max, red, redf);
                 continue;
             }
         }
@@ -2361,8 +2331,7 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     int occ = 0;
     size_t per_cta, cg_smem = 0;
     bool pipe = false;
-    int dense_coarse = 0, sten_threads = kCgStThreads;
-    bool wide = false;
+    int dense_coarse = 0;
     const void *kfn;
     if (o.solver == GC_LINCAL) {
         if (sel->n_ubl > kMaxUbl)
@@ -2383,31 +2352,21 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
             if (dense_coarse) cg_smem += cf;
             else if (cg_smem + cf / 2 <= kCgDnSmem) cg_smem += cf / 2;   // one system: the inversion's scratch
         } else {
-            // stencil operator: while every channel has an SM of its own its
-            // latency is what counts, and arrays of 512 antennas and more take
-            // 512 threads and most of the SM's shared memory for a channel (64
-            // channels of 32x32: 1116 against 1256 us, 16 of 48x48: 1871 against
-            // 2494 us); past that two CTAs of 256 threads per SM have the higher
-            // throughput
-            wide = p.stencil && C <= ctx->sm_count && p.N >= 512;
-            sten_threads = wide ? kCgStMost : kCgStThreads;
-            const size_t cap = wide ? kCgDnSmem - 20480 : kCgSmemMax;
-            cg_smem = cg_arena_bytes(p.N, p.n_ubl, p.L, cap, p.stencil != 0, wide);
-            // pair-scatter operator with its hot vectors in global memory: the pipelined pass
-            pipe = !p.stencil && cg_hot_floats(p.N, p.n_ubl, false) * sizeof(float) > cg_smem;
-            kfn = p.stencil ? (wide ? (const void *)lincal_cg_kernel<false, true, true>
-                                    : (const void *)lincal_cg_kernel<false, true, false>)
-                            : (pipe ? (const void *)lincal_cg_kernel<true, false, false>
-                                    : (const void *)lincal_cg_kernel<false, false, false>);
-            e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
-            if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(lincal_cg)");
+        cg_smem = cg_arena_bytes(p.N, p.n_ubl, p.L, kCgSmemMax, p.stencil != 0);
+        // pair-scatter operator with its hot vectors in global memory: the pipelined pass
+        pipe = !p.stencil && cg_hot_floats(p.N, p.n_ubl, false) * sizeof(float) > cg_smem;
+        kfn = p.stencil ? (const void *)lincal_cg_kernel<false, true>
+                        : (pipe ? (const void *)lincal_cg_kernel<true, false>
+                                : (const void *)lincal_cg_kernel<false, false>);
+        e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
+        if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(lincal_cg)");
         }
     } else {
         per_cta = sizeof(float) * (size_t)(2 * p.N + 2 * p.n_ubl + p.N + 2 * p.N + 2 * p.n_ubl + 64);
         kfn = (const void *)omnical_kernel;
     }
     per_cta = (per_cta + 255) & ~size_t(255);
-    const int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? sten_threads : (p.dense ? kCgDnThreads : kCgThreads)) : kCThreads;
+    const int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? kCgStThreads : (p.dense ? kCgDnThreads : kCgThreads)) : kCThreads;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, nthr, cg_smem);
     if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(calibration)");
     if (ctx->tune[GC_TUNE_CAL_CTAS] > 0) occ = std::min(occ, ctx->tune[GC_TUNE_CAL_CTAS]);
@@ -2425,11 +2384,10 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     int rec = gc_prof_begin(ctx, s, o.solver == GC_LINCAL_CG ? "lincal_cg" : "omnical");
     if (o.solver == GC_LINCAL_CG) {
         const int sf = (int)(cg_smem / sizeof(float));
-        if (wide) lincal_cg_kernel<false, true, true><<<grid, nthr, cg_smem, s>>>(p, 1e-4, 500, sf);
-        else if (p.stencil) lincal_cg_kernel<false, true, false><<<grid, nthr, cg_smem, s>>>(p, 1e-4, 500, sf);
+        if (p.stencil) lincal_cg_kernel<false, true><<<grid, kCgStThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
         else if (p.dense) lincal_cg_dense<<<grid, kCgDnThreads, cg_smem, s>>>(p, 1e-4, 500, sf, dense_coarse);
-        else if (!pipe) lincal_cg_kernel<false, false, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
-        else lincal_cg_kernel<true, false, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
+        else if (!pipe) lincal_cg_kernel<false, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
+        else lincal_cg_kernel<true, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
     } else {
         omnical_kernel<<<grid, kCThreads, 0, s>>>(p);
     }
