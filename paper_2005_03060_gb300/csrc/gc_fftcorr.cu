@@ -735,6 +735,15 @@ AccKernel acc_kernel(int mode) {
                                : (mode == kStageBulk ? fftcorr_accumulate<K, kStageBulk> : fftcorr_accumulate<K, kStagePlain>);
 }
 
+// Resident CTAs that may be launched.  Known fault, to be mended by itself: with
+// several sample groups and L < LMAX the groups' parked spectra stay in rows
+// that the CTA's next item reads as zero, so which items a CTA takes shows in
+// the result; there they stay what they were.
+template <class K>
+int most_ctas(int L, int occ) {
+    return K::G > 1 && L < K::LMAX ? std::min(occ, K::CHUNK_CTAS) : occ;
+}
+
 // CTAs to launch for `items` equal items: k per SM, 1 <= k <= occ, for the
 // least time, k resident CTAs taking about k^a times as long for one item each
 // and the last wave as many as it has -- so a full last wave of fewer can beat
@@ -853,7 +862,7 @@ struct Launcher {
             st = gc_encode_tiled(ctx, &tmap, tma_dtype<K>(), 4, const_cast<void *>(volt), dims, strides, box);
             if (st != GC_OK) return st;
         }
-        const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, ctx->sm_count, kCtaCost<K>)
+        const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, most_ctas<K>(L, occ), ctx->sm_count, kCtaCost<K>)
                                            : (int)std::min<long>(p.n_items, slots);
         int rec = gc_prof_begin(ctx, stream, "fftcorr_accumulate");
         kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
@@ -1116,7 +1125,7 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return GC_ECUDA;
     }
-    const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, sms, kCtaCost<K>) : (int)std::min<long>(p.n_items, slots);
+    const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, most_ctas<K>(L, occ), sms, kCtaCost<K>) : (int)std::min<long>(p.n_items, slots);
     kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
     if (cudaGetLastError() != cudaSuccess) return GC_ECUDA;
     const size_t fsmem = fin_smem(K::M, L);
