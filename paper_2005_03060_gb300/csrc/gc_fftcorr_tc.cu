@@ -71,7 +71,7 @@ constexpr int kRawSamp = kSamp;
 constexpr int kRawStages = 3;
 constexpr int kRawStride = kRawSamp * kTL * kTL + 128;   // + slack for the last row's 8-byte reads
 constexpr int kCoefBytes = kTasks * 8 * kConvThreads * 8;   // [task i][input e][converter thread] float2
-constexpr int kTwBytes = 2 * 2 * 32 * 8;                   // [pr][residue][y] float2
+constexpr int kTwBytes = 2 * 2 * 96 * 4;                   // [pr][residue][table of 16 pairs of y]
 constexpr size_t kSmemTC = (size_t)kBStages * kBStage + (size_t)kRawStages * kRawStride + kCoefBytes + kTwBytes;
 constexpr uint32_t kColD = 0, kColAHi = 256, kColALo = 320, kColP = 384;
 constexpr uint32_t kLBO = 128, kSBO = 2048;   // K-adjacent / N-adjacent core-matrix strides
@@ -86,14 +86,7 @@ struct TcFftParams {
     int n_chunks, n_items;
 };
 
-// multiply by (-i)^R
-template <int R>
-__device__ __forceinline__ float2 rot_mi_tc(float2 a) {
-    if (R == 0) return a;
-    if (R == 1) return make_float2(a.y, -a.x);
-    if (R == 2) return make_float2(-a.x, -a.y);
-    return make_float2(-a.y, a.x);
-}
+constexpr Tw256 kTw = make_tw256();   // the twiddle table for compile-time use
 
 // binary16 hi / lo parts of two floats, packed (lower K index in the low half)
 __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t &lo) {
@@ -104,9 +97,110 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
+// Two FP32 values in a register pair; each lane of the packed operations
+// rounds as the scalar one does.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 p2(float a, float b) {
+    f2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ f2 p2u(uint32_t a, uint32_t b) {
+    f2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ float2 u2(f2 a) {
+    float2 d;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+    return d;
+}
+__device__ __forceinline__ f2 padd(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 psub(f2 a, f2 b) {
+    f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 pmul(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f2 pfma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// One butterfly of the packed FFT: elements u, v of both lanes, v <- (u - v)
+// omega_256^e (the trivial and the eighth-turn twiddles as tw_apply has them).
+template <int E>
+__device__ __forceinline__ void bfly(f2 &ur, f2 &ui, f2 &vr, f2 &vi) {
+    const f2 ar = ur, ai = ui, br = vr, bi = vi;
+    ur = padd(ar, br);
+    ui = padd(ai, bi);
+    if constexpr (E == 0) {
+        vr = psub(ar, br);
+        vi = psub(ai, bi);
+    } else if constexpr (E == 64) {   // times -i: (im, -re)
+        vr = psub(ai, bi);
+        vi = psub(br, ar);
+    } else {
+        const f2 dr = psub(ar, br), di = psub(ai, bi);
+        if constexpr (E == 32 || E == 96) {
+            constexpr float h = 0.70710678118654752f;
+            const f2 hp = p2(h, h), s = padd(dr, di), d = psub(di, dr);
+            vr = pmul(E == 32 ? s : d, hp);
+            vi = E == 32 ? pmul(d, hp) : pmul(s, p2(-h, -h));
+        } else {
+            constexpr float wx = kTw.v[E].x, wy = kTw.v[E].y;
+            vr = pfma(dr, p2(wx, wx), pmul(di, p2(-wy, -wy)));
+            vi = pfma(di, p2(wx, wx), pmul(dr, p2(wy, wy)));
+        }
+    }
+}
+
+// Stages of LEN points over the 16 packed elements (both lanes alike).
+template <int LEN, int I>
+__device__ __forceinline__ void stage(f2 (&r)[16], f2 (&i)[16]) {
+    if constexpr (I < 8) {
+        constexpr int blk = I / (LEN / 2) * LEN, j = I % (LEN / 2);
+        bfly<j * (256 / LEN)>(r[blk + j], i[blk + j], r[blk + j + LEN / 2], i[blk + j + LEN / 2]);
+        stage<LEN, I + 1>(r, i);
+    }
+}
+
+// First stage (32 points): element j with j + 16, in scalar registers -- the
+// results are the two lanes of pack j.
+template <int J>
+__device__ __forceinline__ void first_stage(const float2 (&b)[32], f2 (&r)[16], f2 (&i)[16]) {
+    if constexpr (J < 16) {
+        const float2 u = b[J], v = b[J + 16], d = make_float2(u.x - v.x, u.y - v.y);
+        float2 w;
+        constexpr int E = 8 * J;
+        constexpr float h = 0.70710678118654752f;
+        if constexpr (E == 0) w = d;
+        else if constexpr (E == 64) w = make_float2(d.y, -d.x);
+        else if constexpr (E == 32) w = make_float2((d.x + d.y) * h, (d.y - d.x) * h);
+        else if constexpr (E == 96) w = make_float2((d.y - d.x) * h, -(d.x + d.y) * h);
+        else {
+            constexpr float wx = kTw.v[E].x, wy = kTw.v[E].y;
+            w = make_float2(fmaf(d.x, wx, -(d.y * wy)), fmaf(d.y, wx, d.x * wy));
+        }
+        r[J] = p2(u.x + v.x, w.x);
+        i[J] = p2(u.y + v.y, w.y);
+        first_stage<J + 1>(b, r, i);
+    }
+}
+
 // |X|^2 of one residue's 32 bins into its power columns (first sample of a
-// chunk: stored, later: added), 16 columns at a time
-__device__ __forceinline__ void power_update(const float2 (&b)[32], uint32_t pcol, bool first) {
+// chunk: stored, later: added), 16 columns at a time; bins j and j + 16 of the
+// bit-reversed order sit in columns 2 j and 2 j + 1, the two lanes of pack j.
+__device__ __forceinline__ void power_update(const f2 (&r)[16], const f2 (&i)[16], uint32_t pcol, bool first) {
     if (!first) gc_tmem_wait_st();
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -117,12 +211,16 @@ __device__ __forceinline__ void power_update(const float2 (&b)[32], uint32_t pco
             gc_tmem_ld4_nowait(pcol + 16 * h + 8, pv + 8);
             gc_tmem_ld4_nowait(pcol + 16 * h + 12, pv + 12);
             gc_tmem_wait_ld16_regs(pv);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) pv[k] = 0u;
         }
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float2 v = b[16 * h + i];
-            const float p0 = first ? 0.f : __uint_as_float(pv[i]);
-            pv[i] = __float_as_uint(fmaf(v.x, v.x, fmaf(v.y, v.y, p0)));
+        for (int k = 0; k < 8; ++k) {
+            const f2 X = r[8 * h + k], Y = i[8 * h + k];
+            const float2 o = u2(pfma(X, X, pfma(Y, Y, p2u(pv[2 * k], pv[2 * k + 1]))));
+            pv[2 * k] = __float_as_uint(o.x);
+            pv[2 * k + 1] = __float_as_uint(o.y);
         }
         gc_tmem_st16(pcol + 16 * h, pv);
     }
@@ -130,38 +228,62 @@ __device__ __forceinline__ void power_update(const float2 (&b)[32], uint32_t pco
 
 // The column stage of one sample for the residue pair pr: (0, 2) or (1, 3).
 // For each of the two residues the 64 values X1[k_x][y] of this lane come in
-// with one load of the Re and one of the Im columns (tensor memory is read
-// twice rather than holding both folds in registers); y and y + 32 give the
-// fold input
-//   s2 = pr + 2 h:  (a0 + (-1)^h (-i)^pr a1) omega_128^((pr + 2 h) y)
-// (twiddles from the table tw[h][y]), then a 32-point FFT and |X|^2 -- one
-// copy of the code for both residues and both pairs, so that the
-// instruction cache holds the whole column stage.
+// from tensor memory (read twice rather than holding both folds in registers);
+// y and y + 32 give the fold input
+//   s2 = pr + 2 h:  (a0 + (-1)^h (-i)^pr a1) omega_128^((pr + 2 h) y),
+// then a 32-point FFT and |X|^2.  The arithmetic is packed: neighbouring y share
+// a register pair through fold and twiddles (the rotation (-i)^pr only swaps
+// which columns are loaded as a1's parts), then bins j and j + 16 do, whose
+// remaining stages have the same twiddles.  What bounds the kernel is the FP32
+// pipe and the issue slots of this stage: 256 channels of the 64x64 grid, 8192
+// samples, took 39.5 ms with scalar twiddles and selected columns, 35.8 ms so.
+// (Fetching the powers ahead of the FFT as well made it 0.9 % slower.)  One copy
+// of the code serves both residues and both pairs, so that the instruction
+// cache holds the whole column stage.
+// Twiddle table of a residue: four floats (x, x', y, y') per pair of y, then
+// two (-y, -y').
 __device__ __forceinline__ void column_pair(uint32_t dre, uint32_t dim, uint32_t pcol_a, uint32_t pcol_b,
-                                            bool first, int pr, const float2 *tw) {
+                                            bool first, int pr, const float *tw) {
+    const uint32_t dx = (pr ? dim : dre) + 32, dy = (pr ? dre : dim) + 32;
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
         const float sg = h ? -1.f : 1.f;
-        float2 b[32];
+        const f2 sx = p2(sg, sg), sy = pr ? p2(-sg, -sg) : sx;
+        f2 r[16], i[16];
         {
-            uint32_t re[64], im[64];
-            gc_tmem_ld64_nowait(dre, re);
-            gc_tmem_ld64_nowait(dim, im);
-            gc_tmem_wait_ld();
-            gc_reg_tie32(re);
-            gc_reg_tie32(re + 32);
-            gc_reg_tie32(im);
-            gc_reg_tie32(im + 32);
+            float2 b[32];
+            {
+                uint32_t re[32], im[32], ax[32], ay[32];
+                gc_tmem_ld32_nowait(dre, re);
+                gc_tmem_ld32_nowait(dim, im);
+                gc_tmem_ld32_nowait(dx, ax);
+                gc_tmem_ld32_nowait(dy, ay);
+                gc_tmem_wait_ld();
+                gc_reg_tie32(re);
+                gc_reg_tie32(im);
+                gc_reg_tie32(ax);
+                gc_reg_tie32(ay);
+                const float4 *txy = reinterpret_cast<const float4 *>(tw + 96 * h);
+                const float2 *tn = reinterpret_cast<const float2 *>(tw + 96 * h + 64);
 #pragma unroll
-            for (int y = 0; y < 32; ++y) {
-                const float2 a0 = make_float2(__uint_as_float(re[y]), __uint_as_float(im[y]));
-                const float2 a1 = make_float2(__uint_as_float(re[y + 32]), __uint_as_float(im[y + 32]));
-                const float2 r = pr ? make_float2(a1.y, -a1.x) : a1;   // (-i)^pr a1
-                b[y] = cmul(make_float2(fmaf(sg, r.x, a0.x), fmaf(sg, r.y, a0.y)), tw[32 * h + y]);
+                for (int k = 0; k < 16; ++k) {
+                    const f2 tr = pfma(sx, p2u(ax[2 * k], ax[2 * k + 1]), p2u(re[2 * k], re[2 * k + 1]));
+                    const f2 ti = pfma(sy, p2u(ay[2 * k], ay[2 * k + 1]), p2u(im[2 * k], im[2 * k + 1]));
+                    const float4 w = txy[k];
+                    const float2 n = tn[k];
+                    const float2 x = u2(pfma(tr, p2(w.x, w.y), pmul(ti, p2(n.x, n.y))));
+                    const float2 y = u2(pfma(ti, p2(w.x, w.y), pmul(tr, p2(w.z, w.w))));
+                    b[2 * k] = make_float2(x.x, y.x);
+                    b[2 * k + 1] = make_float2(x.y, y.y);
+                }
             }
+            first_stage<0>(b, r, i);
         }
-        fft_reg<32>(b);
-        power_update(b, h ? pcol_b : pcol_a, first);
+        stage<16, 0>(r, i);
+        stage<8, 0>(r, i);
+        stage<4, 0>(r, i);
+        stage<2, 0>(r, i);
+        power_update(r, i, h ? pcol_b : pcol_a, first);
     }
 }
 
@@ -182,7 +304,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
     unsigned char *bring = smem;
     unsigned char *raw = smem + (size_t)kBStages * kBStage;
     float2 *coef = reinterpret_cast<float2 *>(raw + (size_t)kRawStages * kRawStride);
-    float2 *tws = coef + kCoefBytes / 8;   // column-fold twiddles omega_128^((pr + 2 r) y)
+    float *tws = reinterpret_cast<float *>(coef + kCoefBytes / 8);   // column-fold twiddles omega_128^((pr + 2 r) y)
     __shared__ uint64_t full_raw[kRawStages], empty_raw[kRawStages], full_b[kBStages], empty_b[kBStages];
     __shared__ uint64_t full_d[2], empty_d[2], mma_done;
     __shared__ uint32_t tmem_slot;
@@ -213,7 +335,10 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
     for (int i = tid; i < 2 * 2 * 32; i += kThreadsTC) {
         const int pr = i >> 6, r = (i >> 5) & 1, y = i & 31;
         const cf w = c_tw.v[(2 * (pr + 2 * r) * y) & 255];
-        tws[i] = make_float2(w.x, w.y);
+        float *t = tws + 96 * (2 * pr + r);
+        t[4 * (y >> 1) + (y & 1)] = w.x;
+        t[4 * (y >> 1) + 2 + (y & 1)] = w.y;
+        t[64 + y] = -w.y;
     }
     if (warp == 0) gc_tmem_alloc(&tmem_slot, 512);
     gc_tc_fence_before();
@@ -461,7 +586,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
                 gc_tc_fence_after();
                 const uint32_t dre = lb + kColD + 128 * db, dim = dre + 64;
                 const bool first = s == 0;
-                column_pair(dre, dim, pa, pb, first, pr, tws + 64 * pr);
+                column_pair(dre, dim, pa, pb, first, pr, tws + 192 * pr);
                 gc_tc_fence_before();
                 __syncwarp();
                 if (lane == 0) gc_mbar_arrive(&empty_d[db]);
@@ -481,7 +606,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
                 gc_tmem_ld32_nowait(lb + kColP + 32 * s2, pv);
                 gc_tmem_wait_ld_regs(pv);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) out[(s2 + 4 * bitrev<32>(i)) * kTM + kx] = __uint_as_float(pv[i]);
+                for (int i = 0; i < 32; ++i)   // column 2 j + l holds bin j + 16 l
+                    out[(s2 + 4 * bitrev<32>((i >> 1) + 16 * (i & 1))) * kTM + kx] = __uint_as_float(pv[i]);
             }
         }
         if (!ok) {
