@@ -32,11 +32,11 @@
 //   warps 0-7   column stage: warp w takes tensor-memory lanes 32 (w % 4) ..
 //               +31 and the column residues w / 4 and w / 4 + 2 (one load of
 //               the D columns feeds both folds);
-//   warps 8-9   converters: raw 4+4-bit samples -> w = v / g -> hi / lo
+//   warps 8-11  converters: raw 4+4-bit samples -> w = v / g -> hi / lo
 //               binary16 B operands in shared memory (K-major, no swizzle),
 //               two samples per stage;
-//   warp 10     bulk copies of raw samples (two per stage) into a ring;
-//   warp 11     MMA issue (one thread), completion committed to the rings.
+//   warp 12     bulk copies of raw samples (two per stage) into a ring;
+//   warp 13     MMA issue (one thread), completion committed to the rings.
 // Tensor memory (512 columns): D (two buffers of Re 64 + Im 64 columns),
 // A_hi, A_lo (64 columns each: two binary16 of K per column), the power
 // spectrum (128 columns: 4 residues x 32 bins).  Every wait is bounded; a
@@ -53,15 +53,22 @@ namespace {
 
 constexpr int kTM = 128;                 // FFT side
 constexpr int kTL = 64;                  // largest grid side (rows y and inputs x of the row stage)
-// 12 warps: column stage 0-7 (warp w: tensor-memory lanes 32 (w % 4) .. +31,
+// 16 warps: column stage 0-7 (warp w: tensor-memory lanes 32 (w % 4) .. +31,
 // column residues s2 = (w / 4) and (w / 4) + 2, which share their fold
-// inputs), converters 8-9, bulk copies 10, MMA issue 11.
-constexpr int kThreadsTC = 384;
+// inputs), converters 8-11, one per SM sub-partition beside two column warps,
+// bulk copies 12, MMA issue 13.  (Two converter warps of twelve left two of the
+// four sub-partitions with a third more to issue than the others: 35.8 ms, 33.3
+// with four, 256 channels of the 64x64 grid, 8192 samples.)
+constexpr int kThreadsTC = 512;
+// Registers a thread by warpgroup; two column warpgroups, the converters and the
+// last one together take what the CTA is launched with, 128 a thread.
+constexpr int kColRegs = 168, kConvRegs = 104, kIssueRegs = 72;
+static_assert(2 * kColRegs + kConvRegs + kIssueRegs == 4 * 128, "registers of the four warpgroups");
 constexpr int kEpiWarps = 8;
-constexpr int kWarpConv0 = 8, kConvWarps = 2, kWarpTma = 10, kWarpMma = 11;
+constexpr int kWarpConv0 = 8, kConvWarps = 4, kWarpTma = 12, kWarpMma = 13;
 constexpr int kConvThreads = 32 * kConvWarps;
 constexpr int kTasks = kTL * 8 / kConvThreads;   // (row, group of 8 inputs) tasks per converter thread
-static_assert(kConvWarps == 2 && kTasks == 8, "the converter task map covers 64 rows x 8 input groups with 64 threads");
+static_assert(kConvWarps == 4 && kTasks == 4, "the converter task map covers 64 rows x 8 input groups with 128 threads");
 constexpr int kSamp = 2;                          // samples per raw stage and per B stage
 constexpr int kBStages = 2;
 constexpr int kBPlane = kSamp * kTL * kTM * 2;    // one binary16 B operand of kSamp samples: 32 KB
@@ -374,115 +381,120 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
     __syncthreads();
     gc_tc_fence_after();
     bool ok = true;
-
-    if (warp == kWarpTma) {
-        // ---------------------------------------------------------------- bulk copies of raw samples
-        if (lane == 0) {
-            uint32_t rs = 0, rph = 0;
-            int last_round[kRawStages];
-            for (int i = 0; i < kRawStages; ++i) last_round[i] = -1;
-            int round = 0;
-            for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-                const ItemTC it = decode_tc(p, item);
-                for (int s = 0; s < it.nt; s += kSamp) {
-                    if (!gc_mbar_wait_abort(&empty_raw[rs], rph ^ 1u, &s_abort, GC_WAIT_LIMIT_NS)) {
-                        ok = false;
-                        break;
-                    }
-                    const int ns = min(kSamp, it.nt - s);
-                    const uint32_t bytes = (uint32_t)(ns * N);
-                    gc_mbar_expect_tx(&full_raw[rs], bytes);
-                    gc_bulk_load(raw + (size_t)rs * kRawStride,
-                                 p.volt + ((size_t)it.c * p.T + it.t0 + s) * (size_t)N, bytes, &full_raw[rs]);
-                    last_round[rs] = round;
-                    if (++rs == kRawStages) {
-                        rs = 0;
-                        rph ^= 1u;
-                        ++round;
-                    }
-                }
-            }
-            if (!ok) {
-                s_abort = 1;
-                atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
-            }
-            // no copy may still be landing when the CTA exits
-            for (int i = 0; i < kRawStages; ++i)
-                if (last_round[i] >= 0)
-                    gc_mbar_wait(&full_raw[i], (uint32_t)(last_round[i] & 1), GC_WAIT_LIMIT_NS / 10);
-        }
-        __syncwarp();
-    } else if (warp == kWarpMma) {
-        // ---------------------------------------------------------------- MMA issue
-        if (lane == 0) {
-            const uint32_t idesc = gc_tc_idesc(128, kTL, false, false);
-            const uint32_t bbase = gc_smem_addr(bring);
-            uint32_t bs = 0, bph = 0, db = 0, dph = 0;
-            for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
-                const ItemTC it = decode_tc(p, item);
-                for (int s = 0; s < it.nt && ok; s += kSamp) {
-                    if (!gc_mbar_wait_abort(&full_b[bs], bph, &s_abort, GC_WAIT_LIMIT_NS)) {
-                        ok = false;
-                        break;
-                    }
-                    const int ns = min(kSamp, it.nt - s);
-                    for (int j = 0; j < ns; ++j) {
-                        if (!gc_mbar_wait_abort(&empty_d[db], dph ^ 1u, &s_abort, GC_WAIT_LIMIT_NS)) {
+    // every warp of a warpgroup passes its line
+    if (warp >= kWarpTma) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssueRegs));
+        if (warp == kWarpTma) {
+            // ---------------------------------------------------------------- bulk copies of raw samples
+            if (lane == 0) {
+                uint32_t rs = 0, rph = 0;
+                int last_round[kRawStages];
+                for (int i = 0; i < kRawStages; ++i) last_round[i] = -1;
+                int round = 0;
+                for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+                    const ItemTC it = decode_tc(p, item);
+                    for (int s = 0; s < it.nt; s += kSamp) {
+                        if (!gc_mbar_wait_abort(&empty_raw[rs], rph ^ 1u, &s_abort, GC_WAIT_LIMIT_NS)) {
                             ok = false;
                             break;
                         }
-                        gc_tc_fence_after();
-                        const uint32_t dre = tmem + kColD + 128 * db, dim = dre + 64;
-                        const uint32_t b0 = bbase + (uint32_t)(bs * kBStage + j * kBSample);
-#pragma unroll 1
-                        for (int term = 0; term < 3; ++term) {
-                            const uint32_t a = tmem + (term == 2 ? kColALo : kColAHi);
-                            const uint32_t b = b0 + (term == 1 ? (uint32_t)kBPlane : 0u);
-#pragma unroll
-                            for (int k = 0; k < 8; ++k)
-                                gc_tc_mma_f16_ts(dre, a + 8 * k, gc_tc_sdesc(b + 256 * k, kLBO, kSBO), idesc,
-                                                 (term | k) != 0);
-                            // Im: C with Im w, then -S with Re w
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                gc_tc_mma_f16_ts(dim, a + 8 * k, gc_tc_sdesc(b + 256 * (k + 4), kLBO, kSBO), idesc,
-                                                 (term | k) != 0);
-#pragma unroll
-                            for (int k = 4; k < 8; ++k)
-                                gc_tc_mma_f16_ts(dim, a + 8 * k, gc_tc_sdesc(b + 256 * (k - 4), kLBO, kSBO),
-                                                 idesc | GC_TC_NEGATE_A, 1u);
+                        const int ns = min(kSamp, it.nt - s);
+                        const uint32_t bytes = (uint32_t)(ns * N);
+                        gc_mbar_expect_tx(&full_raw[rs], bytes);
+                        gc_bulk_load(raw + (size_t)rs * kRawStride,
+                                     p.volt + ((size_t)it.c * p.T + it.t0 + s) * (size_t)N, bytes, &full_raw[rs]);
+                        last_round[rs] = round;
+                        if (++rs == kRawStages) {
+                            rs = 0;
+                            rph ^= 1u;
+                            ++round;
                         }
-                        gc_tc_commit(&full_d[db]);
-                        if (++db == 2) {
-                            db = 0;
-                            dph ^= 1u;
-                        }
-                    }
-                    gc_tc_commit(&empty_b[bs]);
-                    if (++bs == kBStages) {
-                        bs = 0;
-                        bph ^= 1u;
                     }
                 }
+                if (!ok) {
+                    s_abort = 1;
+                    atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
+                }
+                // no copy may still be landing when the CTA exits
+                for (int i = 0; i < kRawStages; ++i)
+                    if (last_round[i] >= 0)
+                        gc_mbar_wait(&full_raw[i], (uint32_t)(last_round[i] & 1), GC_WAIT_LIMIT_NS / 10);
             }
-            if (!ok) {
-                s_abort = 1;
-                atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
+            __syncwarp();
+        } else if (warp == kWarpMma) {
+            // ---------------------------------------------------------------- MMA issue
+            if (lane == 0) {
+                const uint32_t idesc = gc_tc_idesc(128, kTL, false, false);
+                const uint32_t bbase = gc_smem_addr(bring);
+                uint32_t bs = 0, bph = 0, db = 0, dph = 0;
+                for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+                    const ItemTC it = decode_tc(p, item);
+                    for (int s = 0; s < it.nt && ok; s += kSamp) {
+                        if (!gc_mbar_wait_abort(&full_b[bs], bph, &s_abort, GC_WAIT_LIMIT_NS)) {
+                            ok = false;
+                            break;
+                        }
+                        const int ns = min(kSamp, it.nt - s);
+                        for (int j = 0; j < ns; ++j) {
+                            if (!gc_mbar_wait_abort(&empty_d[db], dph ^ 1u, &s_abort, GC_WAIT_LIMIT_NS)) {
+                                ok = false;
+                                break;
+                            }
+                            gc_tc_fence_after();
+                            const uint32_t dre = tmem + kColD + 128 * db, dim = dre + 64;
+                            const uint32_t b0 = bbase + (uint32_t)(bs * kBStage + j * kBSample);
+    #pragma unroll 1
+                            for (int term = 0; term < 3; ++term) {
+                                const uint32_t a = tmem + (term == 2 ? kColALo : kColAHi);
+                                const uint32_t b = b0 + (term == 1 ? (uint32_t)kBPlane : 0u);
+    #pragma unroll
+                                for (int k = 0; k < 8; ++k)
+                                    gc_tc_mma_f16_ts(dre, a + 8 * k, gc_tc_sdesc(b + 256 * k, kLBO, kSBO), idesc,
+                                                     (term | k) != 0);
+                                // Im: C with Im w, then -S with Re w
+    #pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    gc_tc_mma_f16_ts(dim, a + 8 * k, gc_tc_sdesc(b + 256 * (k + 4), kLBO, kSBO), idesc,
+                                                     (term | k) != 0);
+    #pragma unroll
+                                for (int k = 4; k < 8; ++k)
+                                    gc_tc_mma_f16_ts(dim, a + 8 * k, gc_tc_sdesc(b + 256 * (k - 4), kLBO, kSBO),
+                                                     idesc | GC_TC_NEGATE_A, 1u);
+                            }
+                            gc_tc_commit(&full_d[db]);
+                            if (++db == 2) {
+                                db = 0;
+                                dph ^= 1u;
+                            }
+                        }
+                        gc_tc_commit(&empty_b[bs]);
+                        if (++bs == kBStages) {
+                            bs = 0;
+                            bph ^= 1u;
+                        }
+                    }
+                }
+                if (!ok) {
+                    s_abort = 1;
+                    atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
+                }
+                // every MMA issued has completed before tensor memory is released
+                gc_tc_commit(&mma_done);
+                gc_mbar_wait(&mma_done, 0, GC_WAIT_LIMIT_NS / 10);
             }
-            // every MMA issued has completed before tensor memory is released
-            gc_tc_commit(&mma_done);
-            gc_mbar_wait(&mma_done, 0, GC_WAIT_LIMIT_NS / 10);
+            __syncwarp();
         }
-        __syncwarp();
     } else if (warp >= kWarpConv0) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kConvRegs));
         // ---------------------------------------------------------------- converters
-        // task i of this thread: row y = 8 i + ((kg + g) & 7), inputs 8 kg ..
-        // 8 kg + 7, with kg = lane & 7 and g = lane / 8 + 4 (converter warp):
+        // task i of this thread: row y = 16 i + 8 (converter warp / 2) + ((kg + g)
+        // & 7), inputs 8 kg .. 8 kg + 7, with kg = lane & 7 and g = lane / 8 + 4
+        // (converter warp):
         // the 8 lanes of a group write 8 different rows of a core-matrix
         // column, so the 16-byte operand stores are free of bank conflicts
         const int ct = tid - 32 * kWarpConv0;
         const int kg = ct & 7;
-        const int ylo = (kg + ((ct & 31) >> 3) + 4 * (ct >> 5)) & 7;
+        const int ylo = 8 * (ct >> 6) + ((kg + (ct >> 3)) & 7);
         uint32_t rs = 0, rph = 0, bs = 0, bph = 0;
         for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
             const ItemTC it = decode_tc(p, item);
@@ -490,7 +502,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
             // antennas, in shared memory that only this thread reads
 #pragma unroll 1
             for (int i = 0; i < kTasks; ++i) {
-                const int y = 8 * i + ylo;
+                const int y = 16 * i + ylo;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const int x = 8 * kg + e;
@@ -517,7 +529,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
                     unsigned char *bhi = bring + (size_t)bs * kBStage + (size_t)j * kBSample, *blo = bhi + kBPlane;
 #pragma unroll 2
                     for (int i = 0; i < kTasks; ++i) {
-                        const int y = 8 * i + ylo;
+                        const int y = 16 * i + ylo;
                         if (y >= L) continue;
                         const uint2 word = *reinterpret_cast<const uint2 *>(rb + y * L + 8 * kg);
                         // n + 8 of the Re and Im nibbles, one byte each
@@ -569,6 +581,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1) fftcorr_tc_accumulate(const TcF
             if (lane == 0) atomicOr(p.status, GC_DEV_TIMEOUT_FFT);
         }
     } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kColRegs));
         // ---------------------------------------------------------------- column stage (warps 0-7)
         const int lq = warp & 3, pr = warp >> 2;
         const int kx = 32 * lq + lane;
@@ -636,6 +649,12 @@ gc_status gc_fft_tc_run(gc_ctx *ctx, const void *volt, int L, int C, int T, cons
     cudaError_t e = cudaFuncSetAttribute(fftcorr_tc_accumulate, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemTC);
     if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(fftcorr_tc_accumulate)");
+    // the warpgroups' shares must not exceed the registers at launch (setmaxnreg.inc would wait for ever)
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, fftcorr_tc_accumulate);
+    if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncGetAttributes(fftcorr_tc_accumulate)");
+    if (fa.numRegs * (kThreadsTC / 128) < 2 * kColRegs + kConvRegs + kIssueRegs)
+        return gc_fail(ctx, GC_EUNSUPPORTED, "fftcorr_tc_accumulate: built with fewer registers than its warps take");
     const int slots = ctx->sm_count;   // one CTA per SM (all 512 tensor-memory columns)
     // time chunks (even lengths) chosen so that the items fill whole waves
     int best_n = 1, best_len = (T + kRawSamp - 1) / kRawSamp * kRawSamp;
