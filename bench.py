@@ -10,8 +10,8 @@ Headline workload (one step = one integration of a 64 x 64 array):
   (V^unique), the reduced X-engine over the subset selection (V^reduced,
   47250 pairs, exact int32), and the per-channel calibration (Gauss-Newton
   lincal with a matrix-free PCG step, FP32 products and FP64 reductions)
-  whose gains the next step's correlator applies.  The banded FP64 and FP32
-  normal-equation solvers and omnical are timed on a channel subset of the
+  whose gains the next step's correlator applies.  The direct solver with
+  FP64 and FP32 gradients and omnical are timed on a channel subset of the
   same V^reduced and reported with their gain difference from the FP64 one.
   The paper-scale complex64 workload (32 x 32 grid, 256 channels, 4096
   samples, 64 x 64 FFT) is measured after it as a secondary line.
@@ -64,13 +64,11 @@ def flops_per_antenna_sample(L: int, M: int) -> float:
     return (10.0 * bfly + 4.0 * M * M + 6.0 * L * L) / (L * L)
 
 
-def lincal_flops_per_iter(N: int, n_ubl: int, P: int, bw: int) -> float:
-    """FP64 flops of one Gauss-Newton iteration of the banded solver:
-    band Cholesky (n bw^2), forward solve of the border and rhs
-    (2 (m+1) n bw), Schur complement (m^2 n), back substitution (2 n bw),
-    assembly (~150 per pair-visit, two visits per pair)."""
-    n, m = 2 * N, 2 * n_ubl
-    return n * bw * bw + 2.0 * (m + 1) * n * bw + m * m * n + 2.0 * n * bw + 300.0 * P
+def lincal_flops_per_iter(P: int) -> float:
+    """FP64 flops of one Gauss-Newton iteration of the direct solver: the
+    gradient and chi^2, 24 FP64 multiply-adds a pair (the step's matrix is
+    factorised in FP32)."""
+    return 48.0 * P
 
 
 def load_peaks():
@@ -538,7 +536,7 @@ def tune_workload(ctx, w) -> dict:
 
 def calibration_variants(w: Workload, Cs: int, reps_fast: int):
     """The other solvers on the first Cs channels of the same V^reduced,
-    compared with the banded FP64 solve (gain difference after the output
+    compared with the direct FP64 solve (gain difference after the output
     convention, which every solver applies)."""
     import numpy as np
     import torch
@@ -891,8 +889,7 @@ def run_ours(args, rank, world, local_rank):
     rl = rooflines(w, kern, st_last, peaks, probes)
     if "lincal_fp64" in variants:
         v64 = variants["lincal_fp64"]
-        D = max(abs(int(dy) * w.L + int(dx)) for dx, dy in w.sel.types.tolist())
-        flops = v64["channels"] * v64["mean_iters"] * lincal_flops_per_iter(w.N, w.sel.n_ubl, w.sel.P, 2 * D + 1)
+        flops = v64["channels"] * v64["mean_iters"] * lincal_flops_per_iter(w.sel.P)
         v64["fp64_frac"] = flops / (v64["ms"] * 1e-3) / 1e12 / probes["fp64"]
     dom = max(kern.items(), key=lambda kv: kv[1][0])[0]
     roofline = dict(rl.get(dom, {"bound": "unknown"}))

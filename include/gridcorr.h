@@ -130,9 +130,10 @@ GC_API int gc_fft_size(int L);
  *   vunique  [C][2L-1][2L-1] c64 (device), index [dy + L - 1][dx + L - 1]
  *   1 <= L <= 128, C >= 1, T >= 1 (GC_EINVAL otherwise); L > 64 (M = 256)
  *   is built for i4c only (GC_EUNSUPPORTED for c64 / c32h).
- * Voltages are staged by TMA when the buffer is 16-byte aligned and a grid
- * row is a multiple of 16 bytes (c64: L even; c32h: L % 4 == 0; i4c:
- * L % 16 == 0), by plain loads otherwise.
+ * Voltages are staged by TMA when the buffer is 16-byte aligned: tiled copies
+ * where a grid row is a multiple of 16 bytes (c64: L even; c32h: L % 4 == 0;
+ * i4c: L % 16 == 0), else bulk copies of whole samples where M >= 64 and they
+ * fit beside the stages; by plain loads otherwise.
  * 4+4-bit voltages on grids of L = 40, 48, 56 or 64 (M = 128, 16-byte
  * aligned, unmasked) take the row stage of the FFT on the tensor cores
  * (tcgen05 kind::f16 products of binary16 hi/lo splits of the DFT matrix and
@@ -285,7 +286,8 @@ GC_API gc_status gc_quantize(gc_ctx *ctx, const float *volt, int C, int T, int N
  *              by default, Sec. 3), FP32; any selection (low-cadence).
  *   GC_LINCAL_CG Gauss-Newton with the step from conjugate gradients on
  *              J^T J, preconditioned by Jacobi plus a patch-level coarse
- *              space, matrix-free (per-antenna gather over the grid, or a
+ *              space, matrix-free (per-antenna gather over the grid, 2-D
+ *              correlations over lag planes for low-cadence selections, or a
  *              scatter over the pair list: "cal.operator"), FP32 products
  *              with FP64 reductions; inexact-Newton CG tolerance
  *              min(0.05, (|grad| / |grad_0|)^(1/4)) relative residual (at
@@ -454,8 +456,10 @@ GC_API gc_status gc_visibility_variance(gc_ctx *ctx, const gc_sel *sel, double s
  *   "cal.ctas_per_sm"  resident calibration CTAs per SM (cap)
  *   "cal.order"        batched work order: 0 largest first, 1 as given
  *   "cal.operator"     GC_LINCAL_CG operator: 0 per-antenna gather over the
- *                      grid (selections of <= 16 baseline-types; others
- *                      fall back to 1), 1 scatter over the pair list
+ *                      grid (selections of <= 16 baseline-types) or lag
+ *                      planes (gc_calibrate, selections that hold a good
+ *                      part of all pairs); others fall back to 1, scatter
+ *                      over the pair list
  *   "xeng.path"        gc_reduce for 4+4-bit voltages: 0 tensor cores where
  *                      they apply, 1 integer SIMT (dp4a), 2 tensor cores only
  *   "xeng.tc_shape"    tensor-core X-engine launch shape (0 default; 1-4:
