@@ -467,7 +467,9 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
 
         // chunk spectrum P[k_y][k_x]: the groups hold the same bins for
         // different samples; groups 1.. park theirs in the (now idle)
-        // intermediate buffer and group 0 adds them up and stores
+        // intermediate buffer and group 0 adds them up and stores.  On a grid
+        // short of the configuration the parked sums lie over rows that the
+        // next item's column pass reads as zero: their reader clears them
         if constexpr (K::G > 1) {
             float *park = reinterpret_cast<float *>(inter);
             if (g > 0) {
@@ -478,7 +480,11 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
             if (g == 0) {
 #pragma unroll
                 for (int i = 0; i < K::F2; ++i)
-                    for (int gg = 1; gg < K::G; ++gg) acc[i] += park[((gg - 1) * K::F2 + i) * K::NCOL + col];
+                    for (int gg = 1; gg < K::G; ++gg) {
+                        float &q = park[((gg - 1) * K::F2 + i) * K::NCOL + col];
+                        acc[i] += q;
+                        if (L < K::LMAX) q = 0.f;
+                    }
             }
         }
         if (g == 0) {
@@ -735,15 +741,6 @@ AccKernel acc_kernel(int mode) {
                                : (mode == kStageBulk ? fftcorr_accumulate<K, kStageBulk> : fftcorr_accumulate<K, kStagePlain>);
 }
 
-// Resident CTAs that may be launched.  Known fault, to be mended by itself: with
-// several sample groups and L < LMAX the groups' parked spectra stay in rows
-// that the CTA's next item reads as zero, so which items a CTA takes shows in
-// the result; there they stay what they were.
-template <class K>
-int most_ctas(int L, int occ) {
-    return K::G > 1 && L < K::LMAX ? std::min(occ, K::CHUNK_CTAS) : occ;
-}
-
 // CTAs to launch for `items` equal items: k per SM, 1 <= k <= occ, for the
 // least time, k resident CTAs taking about k^a times as long for one item each
 // and the last wave as many as it has -- so a full last wave of fewer can beat
@@ -862,7 +859,7 @@ struct Launcher {
             st = gc_encode_tiled(ctx, &tmap, tma_dtype<K>(), 4, const_cast<void *>(volt), dims, strides, box);
             if (st != GC_OK) return st;
         }
-        const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, most_ctas<K>(L, occ), ctx->sm_count, kCtaCost<K>)
+        const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, ctx->sm_count, kCtaCost<K>)
                                            : (int)std::min<long>(p.n_items, slots);
         int rec = gc_prof_begin(ctx, stream, "fftcorr_accumulate");
         kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
@@ -1125,7 +1122,7 @@ gc_status noalloc_run(const NoallocDev &d, const void *volt, int L, int C, int T
             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
         if (r != CUDA_SUCCESS) return GC_ECUDA;
     }
-    const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, most_ctas<K>(L, occ), sms, kCtaCost<K>) : (int)std::min<long>(p.n_items, slots);
+    const int grid = K::CHUNK_CTAS > 0 ? launch_ctas(p.n_items, occ, sms, kCtaCost<K>) : (int)std::min<long>(p.n_items, slots);
     kern<<<grid, K::NTHREADS, smem, stream>>>(tmap, p);
     if (cudaGetLastError() != cudaSuccess) return GC_ECUDA;
     const size_t fsmem = fin_smem(K::M, L);
