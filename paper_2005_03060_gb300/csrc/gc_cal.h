@@ -101,6 +101,13 @@ __device__ void block_sum(R (&v)[NV], R *red /* smem [32][NV] */) {
     __syncthreads();
 }
 
+// Has the channel used up its time?  Thread 0 decides and every thread gets its
+// answer: threads that read the timer for themselves could part in the limit's
+// last instant, some leaving the iteration and some waiting at its barriers.
+__device__ __forceinline__ bool out_of_time(const CalParams &p, uint64_t t_start) {
+    return __syncthreads_or(threadIdx.x == 0 && gc_globaltimer() - t_start > p.deadline_ns) != 0;
+}
+
 // ----------------------------------------------------------------- start point
 // Spanning-tree phases over the (1,0) and (0,1) types (arg V_(1,0) = arg V_(0,1)
 // = 0 fixes the slopes), unit amplitudes, V_alpha = group mean of V_p / (g_i g_j^*).

@@ -1617,7 +1617,7 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
             st = GC_OK;
             break;
         }
-        if (gc_globaltimer() - t_start > p.deadline_ns) {
+        if (out_of_time(p, t_start)) {
             st = GC_ETIMEOUT;
             if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
             break;
@@ -1833,7 +1833,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
                 st = GC_OK;
                 break;
             }
-            if (gc_globaltimer() - t_start > p.deadline_ns) {
+            if (out_of_time(p, t_start)) {
                 st = GC_ETIMEOUT;
                 if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
                 break;
@@ -2115,6 +2115,7 @@ lincal_cg_batched(const __grid_constant__ BatchParams bp) {
 __global__ void __launch_bounds__(kCThreads) omnical_kernel(const CalParams p) {
     __shared__ float red[32 * 2];
     __shared__ double redd[64];
+    __shared__ int s_late;
     float *base = reinterpret_cast<float *>(p.work + (size_t)blockIdx.x * p.work_per_cta);
     float *xg = base;                        // 2N
     float *xv = xg + 2 * p.N;                // 2 n_ubl (+ N scratch for the start point)
@@ -2205,12 +2206,14 @@ __global__ void __launch_bounds__(kCThreads) omnical_kernel(const CalParams p) {
                 acc[1] += (*x) * (*x);
                 *x = (1.f - a) * (*x) + a * xn;
             }
+            // (the time limit's decision shares the sum's barriers)
+            if (threadIdx.x == 0) s_late = gc_globaltimer() - t_start > p.deadline_ns;
             block_sum<float, 2>(acc, red);
             if (sqrtf(acc[0]) < (float)p.tol * sqrtf(acc[1])) {
                 st = GC_OK;
                 break;
             }
-            if (gc_globaltimer() - t_start > p.deadline_ns) {
+            if (s_late) {
                 st = GC_ETIMEOUT;
                 if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
                 break;

@@ -1087,7 +1087,7 @@ __global__ void __launch_bounds__(kLThreads, 1) lincal_kernel(const CalParams p,
                 st = GC_OK;
                 break;
             }
-            if (gc_globaltimer() - t_start > p.deadline_ns) {
+            if (out_of_time(p, t_start)) {
                 st = GC_ETIMEOUT;
                 if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
                 break;
