@@ -1421,6 +1421,68 @@ __device__ void cg_coarse_setup(const CalParams &p, const CgWork &w, float mu) {
     }
 }
 
+// A warm start's zero elements take least-squares values from the others before
+// the first pass.  In relative coordinates a step is a multiple of the element:
+// a visibility or gain of exactly zero has no gradient there and would stay
+// zero, and the channel converge beside its solution.  Visibilities first (each
+// from its type's pairs), then gains (one scan of the pairs for all of them); an
+// element without a pair to take it from stays as it is.
+__device__ void warm_visibilities(const CalParams &p, int c, const CgWork &w) {
+    const float2 *g = reinterpret_cast<const float2 *>(w.xg);
+    float2 *V = reinterpret_cast<float2 *>(w.xv);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int k = wp; k < p.n_ubl; k += nw) {
+        if (V[k].x != 0.f || V[k].y != 0.f) continue;   // (one address: the whole warp agrees)
+        float sx = 0.f, sy = 0.f, sd = 0.f;
+        for (int q = p.type_ptr[k] + lane; q < p.type_ptr[k + 1]; q += 32) {
+            const float2 gi = g[p.pair_i[q]], gj = g[p.pair_j[q]], o = vobs(p, c, q);
+            const float ex = gi.x * gj.x + gi.y * gj.y, ey = gi.y * gj.x - gi.x * gj.y;   // g_i conj(g_j)
+            sx += ex * o.x + ey * o.y;
+            sy += ex * o.y - ey * o.x;
+            sd += ex * ex + ey * ey;
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            sx += __shfl_xor_sync(0xffffffffu, sx, o);
+            sy += __shfl_xor_sync(0xffffffffu, sy, o);
+            sd += __shfl_xor_sync(0xffffffffu, sd, o);
+        }
+        if (lane == 0 && sd > 0.f) V[k] = make_float2(sx / sd, sy / sd);
+    }
+    __syncthreads();
+}
+
+__device__ void warm_gains(const CalParams &p, int c, const CgWork &w) {
+    float2 *g = reinterpret_cast<float2 *>(w.xg);
+    const float2 *V = reinterpret_cast<const float2 *>(w.xv);
+    bool zero = false;
+    for (int i = threadIdx.x; i < p.N; i += blockDim.x) {
+        const bool z = g[i].x == 0.f && g[i].y == 0.f && (!p.mask || p.mask[i]);
+        zero = zero || z;
+        w.b[2 * i] = w.b[2 * i + 1] = 0.f;   // sums of conj(a) o and
+        w.r[i] = z ? 0.f : -1.f;             // |a|^2 (negative: not wanted)
+    }
+    if (!__syncthreads_or(zero)) return;
+    for (int q = threadIdx.x; q < p.P; q += blockDim.x) {
+        const int i = p.pair_i[q], j = p.pair_j[q];
+        const float2 gi = g[i], gj = g[j], v = V[p.pair_type[q]];
+        const bool zi = w.r[i] >= 0.f, zj = w.r[j] >= 0.f;
+        if (zi == zj) continue;   // neither, or no value in the pair
+        const float2 o = vobs(p, c, q);
+        // a = conj(g_j) V, or conj(g_i V) with the conjugate of the pair
+        const float ax = zi ? gj.x * v.x + gj.y * v.y : gi.x * v.x - gi.y * v.y;
+        const float ay = zi ? gj.x * v.y - gj.y * v.x : -(gi.x * v.y + gi.y * v.x);
+        const float oy = zi ? o.y : -o.y;
+        const int m = zi ? i : j;
+        atomicAdd(&w.b[2 * m], ax * o.x + ay * oy);
+        atomicAdd(&w.b[2 * m + 1], ax * oy - ay * o.x);
+        atomicAdd(&w.r[m], ax * ax + ay * ay);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < p.N; i += blockDim.x)
+        if (w.r[i] > 0.f) g[i] = make_float2(w.b[2 * i] / w.r[i], w.b[2 * i + 1] / w.r[i]);
+    __syncthreads();
+}
+
 // One channel of matrix-free Gauss-Newton (used by the per-selection and the
 // batched kernels).  All threads of the CTA call it.  The CG iteration takes
 // four barriers (six with the coarse correction).
@@ -1453,6 +1515,8 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
             w.xv[2 * k + 1] = v.y;
         }
         __syncthreads();
+        warm_visibilities(p, c, w);
+        warm_gains(p, c, w);
     } else {
         start_point<float>(p, c, w.xg, w.xv, redf, w.z);
     }
@@ -1653,6 +1717,8 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
             w.xv[2 * k + 1] = v.y;
         }
         __syncthreads();
+        warm_visibilities(p, c, w);
+        warm_gains(p, c, w);
     } else {
         start_point<float>(p, c, w.xg, w.xv, redf, w.z);
     }
