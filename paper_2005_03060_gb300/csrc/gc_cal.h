@@ -200,16 +200,16 @@ __device__ void start_point(const CalParams &p, int c, R *xg, R *xv, R *red, R *
     __syncthreads();
 }
 
-// chi^2 = sum_p |V_p - g_i g_j^* V_alpha|^2 over all pairs (one visit each)
+// chi^2 = sum_p |so V_p - g_i g_j^* V_alpha|^2 over all pairs (one visit each)
 template <class R>
-__device__ R chi2_of(const CalParams &p, int c, const R *xg, const R *xv, R *red) {
+__device__ R chi2_of(const CalParams &p, int c, const R *xg, const R *xv, R *red, R so = 1) {
     R s[1] = {0};
     for (int q = threadIdx.x; q < p.P; q += blockDim.x) {
         const int i = p.pair_i[q], j = p.pair_j[q], k = p.pair_type[q];
         const float2 v = vobs(p, c, q);
         C2<R> m = cm(cm(C2<R>{xg[2 * i], xg[2 * i + 1]}, cj(C2<R>{xg[2 * j], xg[2 * j + 1]})),
                      C2<R>{xv[2 * k], xv[2 * k + 1]});
-        const R rx = (R)v.x - m.x, ry = (R)v.y - m.y;
+        const R rx = (R)v.x * so - m.x, ry = (R)v.y * so - m.y;
         s[0] += rx * rx + ry * ry;
     }
     block_sum<R, 1>(s, red);

@@ -131,6 +131,22 @@ struct CgWork {
 
 constexpr int kMaxCoarse = 160;
 
+// Powers of two that bring a start point whose gains or visibilities lie far
+// from unity to it, 1 otherwise.  The CG norm is |r|^2 / G with r of the order of
+// |m|^2, the model's fourth power: for visibilities of 1e-12 it would leave FP32's
+// range, and CG would be skipped as if at the solution.  The Levenberg term holds a
+// visibility back by 1e-7 |V|^2 / |g|^2 of its diagonal: from about 1e3 on steps
+// would get short.  Within 2^+-8 (all 4+4-bit data) nothing is scaled and the
+// arithmetic is what it is without.  (Shared memory: registers held through the
+// solve would spill in the gather form.)
+struct UnitScale {
+    float g, v, o;   // what multiplies gains, visibilities and observations
+};
+__device__ __forceinline__ UnitScale &unit_scale() {
+    __shared__ UnitScale u;
+    return u;
+}
+
 __host__ __device__ inline void cg_coarse_dims(int L, int n_ubl, int &B, int &npx, int &ncp, int &nc, int &cv) {
     B = L >= 16 ? L / 8 : (L >= 4 ? 2 : 1);
     npx = (L + B - 1) / B;
@@ -543,7 +559,7 @@ __device__ double rel_resid_pass_t(const CalParams &p, int c, const CgWork &w, b
         const int k = threadIdx.x;
         const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1), W = L - abs(dx);
         s_ra[k] = make_int4(dy * L + dx, dy * W + dx, __ldg(p.type_ptr + k) - max(0, -dy) * W - max(0, -dx), W);
-        s_rb[k] = make_float4(1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)), xv[2 * k], xv[2 * k + 1], 0.f);
+        s_rb[k] = make_float4(unit_scale().o / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)), xv[2 * k], xv[2 * k + 1], 0.f);
     }
     __syncthreads();
     const void *vc = VF == GC_C64 ? (const void *)(reinterpret_cast<const float2 *>(p.vred) + (size_t)c * p.P)
@@ -751,9 +767,9 @@ __device__ float rel_op_pass(const CalParams &p, const CgWork &w, float mu) {
     return curv;
 }
 
-// chi^2 at a trial point (g, V) (global memory), each pair once: the thread
-// owning antenna m takes the pairs (m, m - d_k).
-__device__ float rel_chi2(const CalParams &p, int c, const float *tg, const float *tv, float *red) {
+// chi^2 at a trial point (g, V) (global memory) of the observations times so,
+// each pair once: the thread owning antenna m takes the pairs (m, m - d_k).
+__device__ float rel_chi2(const CalParams &p, int c, const float *tg, const float *tv, float *red, float so) {
     constexpr int KT = kStencilTypes;
     const int L = p.L, nu = p.n_ubl;
     const float2 *g = reinterpret_cast<const float2 *>(tg);
@@ -769,7 +785,7 @@ __device__ float rel_chi2(const CalParams &p, int c, const float *tg, const floa
             const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1);
             const int xj = x - dx, yj = y - dy;
             if (xj < 0 || xj >= L || yj < 0 || yj >= L) continue;
-            const float inv = 1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
+            const float inv = so / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
             const int q = __ldg(p.type_ptr + k) + (yj - max(0, -dy)) * (L - abs(dx)) + (xj - max(0, -dx));
             float ox, oy;
             if (p.vfmt == GC_C64) {
@@ -1022,7 +1038,7 @@ __device__ double dense_resid_pass(const CalParams &p, int c, const CgWork &w, b
     const int2 *vi = reinterpret_cast<const int2 *>(p.vred) + (size_t)c * p.P;
     float *hb = reinterpret_cast<float *>(w.yb);
     for (int k = wp; k < K; k += nw) {
-        const float inv = 1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
+        const float inv = unit_scale().o / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
         const float Vx = xv[2 * k], Vy = xv[2 * k + 1];
         float tx = 0.f, ty = 0.f, td = 0.f;
         const int q1 = __ldg(p.type_ptr + k + 1);
@@ -1451,7 +1467,7 @@ __device__ void warm_visibilities(const CalParams &p, int c, const CgWork &w) {
     __syncthreads();
 }
 
-__device__ void warm_gains(const CalParams &p, int c, const CgWork &w) {
+__device__ void warm_gains(const CalParams &p, int c, const CgWork &w, float so) {
     float2 *g = reinterpret_cast<float2 *>(w.xg);
     const float2 *V = reinterpret_cast<const float2 *>(w.xv);
     bool zero = false;
@@ -1467,7 +1483,9 @@ __device__ void warm_gains(const CalParams &p, int c, const CgWork &w) {
         const float2 gi = g[i], gj = g[j], v = V[p.pair_type[q]];
         const bool zi = w.r[i] >= 0.f, zj = w.r[j] >= 0.f;
         if (zi == zj) continue;   // neither, or no value in the pair
-        const float2 o = vobs(p, c, q);
+        float2 o = vobs(p, c, q);
+        o.x *= so;
+        o.y *= so;
         // a = conj(g_j) V, or conj(g_i V) with the conjugate of the pair
         const float ax = zi ? gj.x * v.x + gj.y * v.y : gi.x * v.x - gi.y * v.y;
         const float ay = zi ? gj.x * v.y - gj.y * v.x : -(gi.x * v.y + gi.y * v.x);
@@ -1516,7 +1534,7 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
         }
         __syncthreads();
         warm_visibilities(p, c, w);
-        warm_gains(p, c, w);
+        warm_gains(p, c, w, 1.f);
     } else {
         start_point<float>(p, c, w.xg, w.xv, redf, w.z);
     }
@@ -1690,6 +1708,38 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
     finish_channel<float>(p, c, w.xg, w.xv, min(it, p.max_iter), st, red, inner);
 }
 
+// Largest component of n floats (NaN is passed over), for the whole CTA.
+__device__ float block_largest(const float *x, int n, float *buf /* [32] */) {
+    float m = 0.f;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmaxf(m, fabsf(x[i]));
+    return block_allreduce(m, true, buf);
+}
+
+__device__ void find_unit_scale(const CgWork &w, float *buf) {
+    const float am = block_largest(w.xg, w.n, buf), vm = block_largest(w.xv, w.m, buf);
+    if (threadIdx.x == 0) {
+        UnitScale &u = unit_scale();
+        u = UnitScale{1.f, 1.f, 1.f};
+        if (am > 0.f && vm > 0.f && isfinite(am) && isfinite(vm)) {
+            const int ea = ilogbf(am), ev = ilogbf(vm);
+            if (abs(ea) > 8 || abs(ev) > 8 || ev - ea > 8)
+                u = UnitScale{ldexpf(1.f, min(126, max(-126, -ea))), ldexpf(1.f, min(126, max(-126, -ev))),
+                              ldexpf(1.f, min(126, max(-126, -2 * ea - ev)))};
+        }
+    }
+    __syncthreads();
+}
+// State times the scale, or over it.
+__device__ void scale_state(const CgWork &w, bool back) {
+    const UnitScale u = unit_scale();
+    if (u.g == 1.f && u.v == 1.f) return;
+    const float sg = back ? 1.f / u.g : u.g, sv = back ? 1.f / u.v : u.v;
+    __syncthreads();
+    for (int i = threadIdx.x; i < w.n; i += blockDim.x) w.xg[i] *= sg;
+    for (int k = threadIdx.x; k < w.m; k += blockDim.x) w.xv[k] *= sv;
+    __syncthreads();
+}
+
 // One channel of matrix-free Gauss-Newton in relative coordinates (the
 // stencil operator, see rel_op_pass, or with kDense the lag-plane operator,
 // see dense_op_pass).  Same outer iteration, forcing terms,
@@ -1718,10 +1768,12 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
         }
         __syncthreads();
         warm_visibilities(p, c, w);
-        warm_gains(p, c, w);
     } else {
         start_point<float>(p, c, w.xg, w.xv, redf, w.z);
     }
+    find_unit_scale(w, redf);
+    scale_state(w, false);
+    if (p.warm) warm_gains(p, c, w, unit_scale().o);
     // coarse index of every element (0xffff: none)
     for (int e = threadIdx.x; e < ne; e += blockDim.x) {
         int ci = -1;
@@ -1887,7 +1939,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
                 }
                 __syncthreads();
                 const float *sg = reinterpret_cast<const float *>(stage);
-                const float ch = kDense ? chi2_of<float>(p, c, sg, sg + 2 * N, redf) : rel_chi2(p, c, sg, sg + 2 * N, redf);
+                const float ch = kDense ? chi2_of<float>(p, c, sg, sg + 2 * N, redf, unit_scale().o) : rel_chi2(p, c, sg, sg + 2 * N, redf, unit_scale().o);
                 if ((double)ch <= chi2 * (1.0 + 1e-6) + 1e-30 || ls == 7) break;
             }
             for (int e = threadIdx.x; e < ne; e += blockDim.x) {
@@ -2063,6 +2115,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
         __syncthreads();
         staged = true;
     }
+    scale_state(w, true);
     finish_channel<float>(p, c, w.xg, w.xv, min(it, p.max_iter), st, red, inner);
 }
 
