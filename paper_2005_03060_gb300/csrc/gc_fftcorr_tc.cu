@@ -45,6 +45,7 @@
 
 #include <algorithm>
 
+#include "gc_f32x2.h"
 #include "gc_fft_reg.h"
 #include "gc_internal.h"
 #include "gc_tcgen05.h"
@@ -102,45 +103,6 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
     const __half2 l = __floats2half2_rn(a - hf.x, b - hf.y);
     hi = *reinterpret_cast<const uint32_t *>(&h);
     lo = *reinterpret_cast<const uint32_t *>(&l);
-}
-
-// Two FP32 values in a register pair; each lane of the packed operations
-// rounds as the scalar one does.
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 p2(float a, float b) {
-    f2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
-    return d;
-}
-__device__ __forceinline__ f2 p2u(uint32_t a, uint32_t b) {
-    f2 d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ float2 u2(f2 a) {
-    float2 d;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
-    return d;
-}
-__device__ __forceinline__ f2 padd(f2 a, f2 b) {
-    f2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 psub(f2 a, f2 b) {
-    f2 d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 pmul(f2 a, f2 b) {
-    f2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ f2 pfma(f2 a, f2 b, f2 c) {
-    f2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
 }
 
 // One butterfly of the packed FFT: elements u, v of both lanes, v <- (u - v)

@@ -9,69 +9,75 @@
 // does not depend on the launch.
 #include <algorithm>
 
+#include "gc_f32x2.h"
 #include "gc_internal.h"
 
 namespace {
 
 constexpr int kQThreads = 256;
 
-// Running sum of squares as an unevaluated pair s + c of floats: the product
-// x x as p + e (e its exact rounding error, by fma), then the exact two-term
-// sum of s and p (Knuth), with every rounding error collected in c.  About 44
-// bits, ten FP32 operations a component.
-struct Sum2 {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void square(float x) {
-        const float p = __fmul_rn(x, x), e = __fmaf_rn(x, x, -p);
-        const float t = __fadd_rn(s, p), b = __fsub_rn(t, s);
-        c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(p, b)), e));
-        s = t;
+// Running sums of squares of two neighbouring components as unevaluated triples
+// s + c + d of floats.  The product x x is p + e (e its exact rounding error, by
+// fma); p is added to s by the exact two-term sum (Knuth), its error and e to c
+// likewise, and only what is left of those is rounded, in d: about 66 bits, more
+// than an FP64 sum keeps.  (A pair s + c rounds e away: the low bits of squares
+// are not symmetric, and sums came out 6e-16 low.)  Packed: 24 operations for two.
+struct Sum3 {
+    f2 s = 0, c = 0, d = 0;
+    // a + b = t + the value returned
+    static __device__ __forceinline__ f2 two_sum(f2 a, f2 b, f2 &t) {
+        t = padd(a, b);
+        const f2 z = psub(t, a);
+        return padd(psub(a, psub(t, z)), psub(b, z));
+    }
+    __device__ __forceinline__ void square(float x0, float x1) {
+        const float2 q = make_float2(__fmul_rn(x0, x0), __fmul_rn(x1, x1));
+        const f2 p = p2(q.x, q.y), e = p2(__fmaf_rn(x0, x0, -q.x), __fmaf_rn(x1, x1, -q.y));
+        const f2 r = two_sum(c, two_sum(s, p, s), c);
+        d = padd(d, padd(two_sum(c, e, c), r));
+    }
+    __device__ __forceinline__ double value() const {
+        const float2 x = u2(s), y = u2(c), z = u2(d);
+        return ((double)x.x + ((double)y.x + z.x)) + ((double)x.y + ((double)y.y + z.y));
     }
 };
 
-// Squares summed per thread in float pairs, the threads' sums in FP64.  An
-// FP64 fma of every component is bound by this part's FP64 rate (1.05 TFLOP/s,
-// 1/74 of FP32): 1117 us for 64 channels of 2048 x 1024 voltages (1.07 GB)
-// against 212 us for the pairs (5.1 TB/s), which the HBM read bounds.  Four loads a
-// thread are in flight.
-__global__ void __launch_bounds__(kQThreads)
+// Each thread sums its squares in such triples, the threads' sums are added in
+// FP64: rms error of a thread's sum of 256 squares 4e-17, 1e-15 with FP64
+// additions.  An FP64 fma of every component is bound by this part's FP64 rate (1.05
+// TFLOP/s, 1/74 of FP32): the whole quantiser takes 1357 us with it on 64 channels
+// of 2048 x 1024 voltages (1.07 GB), 435 us so, near the HBM reads of both passes
+// (109 and 53 us on a sixteenth of that, in L2, where the FP32 issue bounds it).
+// Four loads a thread are in flight; four CTAs an SM leave the registers for them (435 us;
+// 452 at three, 472 at five, which spills).
+__global__ void __launch_bounds__(kQThreads, 4)
 quant_sumsq(const float4 *__restrict__ v, size_t n4_per_ch, int nblk, double *__restrict__ part) {
     const int c = blockIdx.y, b = blockIdx.x;
     const float4 *src = v + (size_t)c * n4_per_ch;
     const size_t per = (n4_per_ch + nblk - 1) / nblk;
     const size_t lo = min(n4_per_ch, (size_t)b * per), hi = min(n4_per_ch, lo + per);
     constexpr int U = 4;
-    Sum2 acc[4];   // one per component of the float4: independent chains
+    Sum3 xy, zw;
+    unsigned bits = 0u;   // of all values: 0 or the sign alone when all are zero
+    auto take = [&](float4 q) {
+        xy.square(q.x, q.y);
+        zw.square(q.z, q.w);
+        bits |= __float_as_uint(q.x) | __float_as_uint(q.y);
+        bits |= __float_as_uint(q.z) | __float_as_uint(q.w);
+    };
     size_t i = lo + threadIdx.x;
     for (; i + (U - 1) * kQThreads < hi; i += U * kQThreads) {
         float4 q[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) q[u] = src[i + u * kQThreads];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            acc[0].square(q[u].x);
-            acc[1].square(q[u].y);
-            acc[2].square(q[u].z);
-            acc[3].square(q[u].w);
-        }
+        for (int u = 0; u < U; ++u) take(q[u]);
     }
-    for (; i < hi; i += kQThreads) {
-        const float4 q = src[i];
-        acc[0].square(q.x);
-        acc[1].square(q.y);
-        acc[2].square(q.z);
-        acc[3].square(q.w);
-    }
-    double s = 0.0;
-    bool fine = true;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        // squares near the ends of FP32's range (|x| above 1e17 or all below
-        // 1e-12, zeros and non-finite values among them) are summed in FP64
-        fine = fine && acc[k].s > 1e-24f && acc[k].s < 1e34f;
-        s += (double)acc[k].s + (double)acc[k].c;
-    }
-    if (!fine) {
+    for (; i < hi; i += kQThreads) take(src[i]);
+    double s = xy.value() + zw.value();
+    // sums near the ends of FP32's range (|x| above 1e17 or all below 1e-12,
+    // non-finite values among them) are made in FP64; zeros are what they are
+    if (!(s > 1e-24 && s < 1e34) && (bits & 0x7fffffffu) != 0u) {
         s = 0.0;
         for (size_t k = lo + threadIdx.x; k < hi; k += kQThreads) {
             const float4 q = src[k];
