@@ -71,18 +71,36 @@ void fill_pairs(gc_sel *s) {
     s->pair_i.clear();
     s->pair_j.clear();
     s->pair_type.clear();
+    if (!s->masked) {   // whole rectangles: sizes known, rows of consecutive antennas
+        size_t total = 0;
+        for (int k = 0; k < s->n_ubl; ++k) total += (size_t)group_size(L, {s->types[2 * k], s->types[2 * k + 1]});
+        s->pair_i.resize(total);
+        s->pair_j.resize(total);
+        s->pair_type.resize(total);
+    }
+    size_t at = 0;
     for (int k = 0; k < s->n_ubl; ++k) {
-        const int dx = s->types[2 * k], dy = s->types[2 * k + 1];
-        for (int y = 0; y < L; ++y)
-            for (int x = 0; x < L; ++x) {
-                const int xi = x + dx, yi = y + dy;
-                if (xi < 0 || xi >= L || yi < 0 || yi >= L) continue;
-                if (s->masked && !(s->mask[yi * L + xi] && s->mask[y * L + x])) continue;
-                s->pair_i.push_back(yi * L + xi);
-                s->pair_j.push_back(y * L + x);
-                s->pair_type.push_back(k);
+        const int dx = s->types[2 * k], dy = s->types[2 * k + 1], d = dy * L + dx;
+        const int x0 = std::max(0, -dx), x1 = std::min(L, L - dx);
+        for (int y = std::max(0, -dy); y < std::min(L, L - dy); ++y) {
+            if (s->masked) {
+                for (int j = y * L + x0; j < y * L + x1; ++j) {
+                    if (!(s->mask[j + d] && s->mask[j])) continue;
+                    s->pair_i.push_back(j + d);
+                    s->pair_j.push_back(j);
+                    s->pair_type.push_back(k);
+                }
+                continue;
             }
-        s->type_ptr.push_back((int32_t)s->pair_i.size());
+            int32_t *pi = s->pair_i.data() + at, *pj = s->pair_j.data() + at, *pt = s->pair_type.data() + at;
+            for (int x = 0; x < x1 - x0; ++x) {
+                pi[x] = y * L + x0 + d + x;
+                pj[x] = y * L + x0 + x;
+                pt[x] = k;
+            }
+            at += x1 - x0;
+        }
+        s->type_ptr.push_back(s->masked ? (int32_t)s->pair_i.size() : (int32_t)at);
     }
     s->P = (int)s->pair_i.size();
     // (on a full grid only omnical reads it, and for many types arithmetic is
@@ -107,24 +125,33 @@ void fill_pairs(gc_sel *s) {
 // whole groups while it holds every j mod 16; the rest is matched across
 // classes, first fit.  (In type order a group spans two grid rows of its type's
 // rectangle and a 32x32 array pays 1.47 reads for each; in this order 1.04.)
-void order_entries(const gc_sel *s, std::vector<int32_t> &q, std::vector<int32_t> &out) {
+// The class is one of the type, so that a counting sort with a table of j mod 16
+// does without arithmetic on the pairs.
+// types: the window's `nt` types; by: room for its pairs; returns past the last entry.
+int32_t *order_entries(const gc_sel *s, const unsigned char *mod16, const int32_t *types, int nt, int32_t *by, int32_t *out) {
     int n[257] = {0}, at[256];
-    const int pad = gc_xeng_pairs_pitch(s->L) - s->L;
-    auto slot = [&](int e) {
-        const int i = s->pair_i[e] + pad * (s->pair_i[e] / s->L), j = s->pair_j[e] + pad * (s->pair_j[e] / s->L);
-        return (((i - j) & 15) << 4) | (j & 15);
-    };
-    for (int e : q) ++n[slot(e) + 1];
+    const int pitch = gc_xeng_pairs_pitch(s->L);
+    auto cls = [&](int k) { return 16 * ((s->types[2 * k + 1] * pitch + s->types[2 * k]) & 15); };
+    for (int t = 0; t < nt; ++t) {
+        int *m = n + 1 + cls(types[t]);
+        for (int q = s->type_ptr[types[t]]; q < s->type_ptr[types[t] + 1]; ++q) ++m[mod16[s->pair_j[q]]];
+    }
     for (int b = 0; b < 256; ++b) n[b + 1] += n[b];
     std::copy(n, n + 256, at);
-    std::vector<int32_t> by(q.size());
-    for (int e : q) by[at[slot(e)]++] = e;
+    for (int t = 0; t < nt; ++t) {
+        int *m = at + cls(types[t]);
+        for (int q = s->type_ptr[types[t]]; q < s->type_ptr[types[t] + 1]; ++q) by[m[mod16[s->pair_j[q]]]++] = q;
+    }
     std::copy(n, n + 256, at);
     for (int c = 0; c < 16; ++c) {
         int whole = n[16 * c + 1] - n[16 * c];
         for (int r = 1; r < 16; ++r) whole = std::min(whole, n[16 * c + r + 1] - n[16 * c + r]);
-        for (int k = 0; k < whole; ++k)
-            for (int r = 0; r < 16; ++r) out.push_back(by[at[16 * c + r]++]);
+        for (int r = 0; r < 16; ++r) {
+            const int32_t *from = by + at[16 * c + r];
+            for (int k = 0; k < whole; ++k) out[16 * k + r] = from[k];
+            at[16 * c + r] += whole;
+        }
+        out += 16 * whole;
     }
     unsigned has[16] = {0};   // classes left per j mod 16
     size_t left = 0;
@@ -136,7 +163,7 @@ void order_entries(const gc_sel *s, std::vector<int32_t> &q, std::vector<int32_t
         }
     auto take = [&](int c, int r) {
         const int b = 16 * c + r;
-        out.push_back(by[at[b]++]);
+        *out++ = by[at[b]++];
         if (at[b] == n[b + 1]) has[r] &= ~(1u << c);
         --left;
     };
@@ -163,6 +190,7 @@ void order_entries(const gc_sel *s, std::vector<int32_t> &q, std::vector<int32_t
                 ++got;
             }
     }
+    return out;
 }
 
 // X-engine work groups: types that share a window, at most GC_XENG_NTY each.
@@ -208,22 +236,27 @@ void fill_groups(gc_sel *s) {
     s->wp_t1.clear();
     const int N = s->L * s->L;
     if (s->n_windows < 2 || N > 25600) return;   // larger grids do not fit its stages in any format
-    s->wp_entry.reserve((size_t)s->P + (size_t)s->n_windows * N);
+    s->wp_entry.resize((size_t)s->P + (size_t)s->n_windows * N);
     s->wp_off.push_back(0);
-    std::vector<int32_t> win;
-    for (int g = 0; g < s->n_groups; ++g) {
+    std::vector<unsigned char> mod16(N);   // staged position of an antenna, modulo 16
+    for (int j = 0; j < N; ++j) mod16[j] = (unsigned char)((j + (gc_xeng_pairs_pitch(s->L) - s->L) * (j / s->L)) & 15);
+    std::vector<int32_t> by;
+    int32_t *out = s->wp_entry.data();
+    for (int g = 0, g0 = 0; g < s->n_groups; ++g) {
         if (s->grp_first[g]) {
             s->wp_t0.push_back(s->grp_t0[g]);
             s->wp_t1.push_back(s->grp_t1[g]);
-            win.clear();
+            g0 = g;
         }
-        for (int o = s->grp_off[g]; o < s->grp_off[g + 1]; ++o)
-            for (int q = s->type_ptr[s->grp_types[o]]; q < s->type_ptr[s->grp_types[o] + 1]; ++q) win.push_back(q);
-        if (g + 1 == s->n_groups || s->grp_first[g + 1]) {   // the window's last group
-            order_entries(s, win, s->wp_entry);
-            for (int j = 0; j < N; ++j) s->wp_entry.push_back(s->P + j);
-            s->wp_off.push_back((int32_t)s->wp_entry.size());
-        }
+        if (g + 1 < s->n_groups && !s->grp_first[g + 1]) continue;   // not the window's last group
+        const int32_t *types = s->grp_types.data() + s->grp_off[g0];
+        const int nt = s->grp_off[g + 1] - s->grp_off[g0];
+        size_t pairs = 0;
+        for (int t = 0; t < nt; ++t) pairs += s->type_ptr[types[t] + 1] - s->type_ptr[types[t]];
+        if (by.size() < pairs) by.resize(pairs);
+        out = order_entries(s, mod16.data(), types, nt, by.data(), out);
+        for (int j = 0; j < N; ++j) *out++ = s->P + j;
+        s->wp_off.push_back((int32_t)(out - s->wp_entry.data()));
     }
 }
 
@@ -297,8 +330,9 @@ bool fill_tree(gc_sel *s) {
 }
 
 // Largest selection the builders hold: 2^28 pairs (3.2 GB of host pair
-// arrays, as much again on the device).  Low-cadence selections take every
-// pair, N (N - 1) / 2, so they stop at about 23 000 antennas.
+// arrays, with several windows 1.1 GB of entry lists, as much again on the
+// device).  Low-cadence selections take every pair, N (N - 1) / 2, so they stop
+// at about 23 000 antennas.
 constexpr long kMaxPairs = 1L << 28;
 
 // No C++ exception leaves the C ABI: allocation failure reads GC_ENOMEM.
