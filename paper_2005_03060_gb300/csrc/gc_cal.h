@@ -101,11 +101,12 @@ __device__ void block_sum(R (&v)[NV], R *red /* smem [32][NV] */) {
     __syncthreads();
 }
 
-// Has the channel used up its time?  Thread 0 decides and every thread gets its
-// answer: threads that read the timer for themselves could part in the limit's
-// last instant, some leaving the iteration and some waiting at its barriers.
+// Has the channel used up its time?  One thread asks, ahead of a barrier that the
+// iteration has anyway, and all threads read its answer after it: threads that
+// read the timer for themselves could part in the limit's last instant, some
+// leaving the iteration and some waiting at its barriers.
 __device__ __forceinline__ bool out_of_time(const CalParams &p, uint64_t t_start) {
-    return __syncthreads_or(threadIdx.x == 0 && gc_globaltimer() - t_start > p.deadline_ns) != 0;
+    return gc_globaltimer() - t_start > p.deadline_ns;
 }
 
 // ----------------------------------------------------------------- start point

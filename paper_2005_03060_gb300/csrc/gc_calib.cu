@@ -559,7 +559,8 @@ __device__ double rel_resid_pass_t(const CalParams &p, int c, const CgWork &w, b
         const int k = threadIdx.x;
         const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1), W = L - abs(dx);
         s_ra[k] = make_int4(dy * L + dx, dy * W + dx, __ldg(p.type_ptr + k) - max(0, -dy) * W - max(0, -dx), W);
-        s_rb[k] = make_float4(unit_scale().o / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)), xv[2 * k], xv[2 * k + 1], 0.f);
+        s_rb[k] = make_float4(unit_scale().o * (1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k))), xv[2 * k],
+                              xv[2 * k + 1], 0.f);
     }
     __syncthreads();
     const void *vc = VF == GC_C64 ? (const void *)(reinterpret_cast<const float2 *>(p.vred) + (size_t)c * p.P)
@@ -785,7 +786,7 @@ __device__ float rel_chi2(const CalParams &p, int c, const float *tg, const floa
             const int dx = __ldg(p.types + 2 * k), dy = __ldg(p.types + 2 * k + 1);
             const int xj = x - dx, yj = y - dy;
             if (xj < 0 || xj >= L || yj < 0 || yj >= L) continue;
-            const float inv = so / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
+            const float inv = so * (1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)));
             const int q = __ldg(p.type_ptr + k) + (yj - max(0, -dy)) * (L - abs(dx)) + (xj - max(0, -dx));
             float ox, oy;
             if (p.vfmt == GC_C64) {
@@ -1038,7 +1039,7 @@ __device__ double dense_resid_pass(const CalParams &p, int c, const CgWork &w, b
     const int2 *vi = reinterpret_cast<const int2 *>(p.vred) + (size_t)c * p.P;
     float *hb = reinterpret_cast<float *>(w.yb);
     for (int k = wp; k < K; k += nw) {
-        const float inv = unit_scale().o / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k));
+        const float inv = unit_scale().o * (1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)));
         const float Vx = xv[2 * k], Vy = xv[2 * k + 1];
         float tx = 0.f, ty = 0.f, td = 0.f;
         const int q1 = __ldg(p.type_ptr + k + 1);
@@ -1518,6 +1519,7 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
     gw.n = w.n;
     gw.m = w.m;
     __shared__ float sbuf[2 * 32 * kFastSumMax];
+    __shared__ int s_late;
     int par = 0;
     const bool coarse = nc > 0;
     const uint64_t t_start = gc_globaltimer();
@@ -1694,12 +1696,13 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
             if (i < w.n) w.xg[i] = w.trial[i];
             else w.xv[i - w.n] = w.trial[i];
         }
+        if (threadIdx.x == 0) s_late = out_of_time(p, t_start);
         __syncthreads();
         if ((double)step * sqrt(nr[1]) <= p.tol * sqrt(nr[0])) {
             st = GC_OK;
             break;
         }
-        if (out_of_time(p, t_start)) {
+        if (s_late) {
             st = GC_ETIMEOUT;
             if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
             break;
@@ -1708,23 +1711,33 @@ __device__ void cg_solve_channel(const CalParams &p, int c, CgWork &w, double cg
     finish_channel<float>(p, c, w.xg, w.xv, min(it, p.max_iter), st, red, inner);
 }
 
-// Largest component of n floats (NaN is passed over), for the whole CTA.
-__device__ float block_largest(const float *x, int n, float *buf /* [32] */) {
-    float m = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmaxf(m, fabsf(x[i]));
-    return block_allreduce(m, true, buf);
-}
-
-__device__ void find_unit_scale(const CgWork &w, float *buf) {
-    const float am = block_largest(w.xg, w.n, buf), vm = block_largest(w.xv, w.m, buf);
-    if (threadIdx.x == 0) {
-        UnitScale &u = unit_scale();
-        u = UnitScale{1.f, 1.f, 1.f};
-        if (am > 0.f && vm > 0.f && isfinite(am) && isfinite(vm)) {
-            const int ea = ilogbf(am), ev = ilogbf(vm);
-            if (abs(ea) > 8 || abs(ev) > 8 || ev - ea > 8)
-                u = UnitScale{ldexpf(1.f, min(126, max(-126, -ea))), ldexpf(1.f, min(126, max(-126, -ev))),
-                              ldexpf(1.f, min(126, max(-126, -2 * ea - ev)))};
+// The scale of the start point, from the largest components of its gains and
+// visibilities (as bits, whose order is that of the absolute values).
+__device__ void find_unit_scale(const CgWork &w, float *buf /* [64] */) {
+    unsigned *top = reinterpret_cast<unsigned *>(buf);
+    unsigned a = 0u, v = 0u;
+    for (int i = threadIdx.x; i < w.n; i += blockDim.x) a = max(a, __float_as_uint(w.xg[i]) & 0x7fffffffu);
+    for (int k = threadIdx.x; k < w.m; k += blockDim.x) v = max(v, __float_as_uint(w.xv[k]) & 0x7fffffffu);
+    a = __reduce_max_sync(0xffffffffu, a);
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) {
+        top[threadIdx.x >> 5] = a;
+        top[32 + (threadIdx.x >> 5)] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const bool in = threadIdx.x < blockDim.x / 32;
+        const float am = __uint_as_float(__reduce_max_sync(0xffffffffu, in ? top[threadIdx.x] : 0u));
+        const float vm = __uint_as_float(__reduce_max_sync(0xffffffffu, in ? top[32 + threadIdx.x] : 0u));
+        if (threadIdx.x == 0) {
+            UnitScale u{1.f, 1.f, 1.f};
+            if (am > 0.f && vm > 0.f && isfinite(am) && isfinite(vm)) {
+                const int ea = ilogbf(am), ev = ilogbf(vm);
+                if (abs(ea) > 8 || abs(ev) > 8 || ev - ea > 8)
+                    u = UnitScale{ldexpf(1.f, min(126, max(-126, -ea))), ldexpf(1.f, min(126, max(-126, -ev))),
+                                  ldexpf(1.f, min(126, max(-126, -2 * ea - ev)))};
+            }
+            unit_scale() = u;
         }
     }
     __syncthreads();
@@ -1752,6 +1765,7 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
                                      float *redf) {
     const int ne = p.N + p.n_ubl, L = p.L, nc = w.nc, N = p.N;
     __shared__ float sbuf[2 * 32 * kFastSumMax];
+    __shared__ int s_late;
     int par = 0;
     const bool coarse = nc > 0;
     const uint64_t t_start = gc_globaltimer();
@@ -1946,12 +1960,13 @@ __device__ void cg_solve_channel_rel(const CalParams &p, int c, CgWork &w, doubl
                 if (e < N) reinterpret_cast<float2 *>(w.xg)[e] = stage[e];
                 else reinterpret_cast<float2 *>(w.xv)[e - N] = stage[e];
             }
+            if (threadIdx.x == 0) s_late = out_of_time(p, t_start);
             __syncthreads();
             if ((double)step * sqrt(nr[1]) <= p.tol * sqrt(nr[0])) {
                 st = GC_OK;
                 break;
             }
-            if (out_of_time(p, t_start)) {
+            if (s_late) {
                 st = GC_ETIMEOUT;
                 if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
                 break;
@@ -2325,8 +2340,7 @@ __global__ void __launch_bounds__(kCThreads) omnical_kernel(const CalParams p) {
                 acc[1] += (*x) * (*x);
                 *x = (1.f - a) * (*x) + a * xn;
             }
-            // (the time limit's decision shares the sum's barriers)
-            if (threadIdx.x == 0) s_late = gc_globaltimer() - t_start > p.deadline_ns;
+            if (threadIdx.x == 0) s_late = out_of_time(p, t_start);   // (the sum has barriers)
             block_sum<float, 2>(acc, red);
             if (sqrtf(acc[0]) < (float)p.tol * sqrtf(acc[1])) {
                 st = GC_OK;

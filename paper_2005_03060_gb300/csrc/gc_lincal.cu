@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(kLThreads, 1) lincal_kernel(const CalParams p,
     __shared__ double redd2[16 * 12 + 32];
     __shared__ double redd[64];
     __shared__ LinTypes ty;
-    __shared__ int s_fail[2];
+    __shared__ int s_fail[2], s_late;
     const int N = p.N, K = p.n_ubl, L = p.L, nt = blockDim.x, ne = N + K;
     const int hn = nt / 2, sys = threadIdx.x >= hn ? 1 : 0, ht = threadIdx.x - sys * hn;
     LinWork<R> w;
@@ -1070,6 +1070,7 @@ __global__ void __launch_bounds__(kLThreads, 1) lincal_kernel(const CalParams p,
             // halving line search on chi^2; the pass that tries a point is
             // also the next iteration's gradient there
             R step = 1, c2 = 0;
+            if (threadIdx.x == 0) s_late = out_of_time(p, t_start);   // (lin_resid has barriers)
             for (int ls = 0;; ++ls) {
                 c2 = lin_resid<R>(p, c, w.tr, w, ty, red);
                 if (c2 <= chi2 * (1 + kRise) + (R)1e-30 || ls == 7) break;
@@ -1087,7 +1088,7 @@ __global__ void __launch_bounds__(kLThreads, 1) lincal_kernel(const CalParams p,
                 st = GC_OK;
                 break;
             }
-            if (out_of_time(p, t_start)) {
+            if (s_late) {
                 st = GC_ETIMEOUT;
                 if (threadIdx.x == 0) atomicOr(p.status, GC_DEV_TIMEOUT_CAL);
                 break;
