@@ -826,6 +826,11 @@ __device__ float rel_chi2(const CalParams &p, int c, const float *tg, const floa
 constexpr int kCgDnThreads = 512;
 __host__ __device__ inline int dense_lag_row(int L) { return (2 * L - 1 + 7) / 8 * 8; }
 __host__ __device__ inline int dense_row(int L) { return 3 * L + 5; }
+// threads that the wider of both sums needs at least (one per task, below)
+__host__ __device__ inline int dense_tasks(int L) {
+    const int a = L * ((L + 7) / 8), b = (L / 2 + 1) * (dense_lag_row(L) / 8);
+    return a > b ? a : b;
+}
 __host__ __device__ inline size_t cg_dense_floats(int L) {
     const size_t W = 2 * L - 1, plane = (W * W + 8 + 3) / 4 * 4, E = ((size_t)L * dense_row(L) + 3) / 4 * 4;
     return plane + 2 * plane + 2 * E + E + 2 * (((size_t)L * L + 1) / 2 * 2) + 2 * (size_t)L * dense_lag_row(L);
@@ -845,7 +850,6 @@ __device__ void dense_layout(const CalParams &p, CgWork &w, float *at) {
 __device__ void dense_antenna_sums(const CalParams &p, const CgWork &w) {
     const int L = p.L, W = 2 * L - 1, Ew = dense_row(L);
     const int nseg = (L + 7) / 8, tasks = L * nseg, S = min(L, max(1, (int)blockDim.x / tasks));
-    // (tasks <= blockDim.x: L <= 64)
     const int task = threadIdx.x % tasks, split = threadIdx.x / tasks;
     const int y = task / nseg, x0 = 8 * (task - y * nseg);
     float2 acc[8];
@@ -2401,11 +2405,14 @@ static gc_status fill_params(gc_ctx *ctx, gc_sel *sel, int C, const void *vreduc
     // both full-grid selection builders take baseline-types whole, in
     // pair_index order; a partly occupied lattice takes the pair-list form
     p.stencil = ctx->tune[GC_TUNE_CAL_OP] == 0 && sel->n_ubl <= kStencilTypes && !sel->masked ? 1 : 0;
-    // the lag planes: many types, at least a sixteenth of all pairs (the pair
-    // scatter costs 2.9 cycles a pair and SM, the planes 0.08 a product of
-    // antennas: the lines cross at a thirty-eighth), and planes that fit beside the vectors
+    // the lag planes: many types, at least a sixteenth of all pairs, a thread per
+    // task, and planes that fit beside the vectors.  At a sixteenth (subsets of
+    // two and four times the usual pair count) they take 1.29 against 1.54 ms for 64
+    // channels of 16x16 antennas, 2.3 against 3.8 for 24x24; below it, where the
+    // cost of a pair and of a product of antennas let the lines cross at about a
+    // thirty-eighth, nothing was timed and the scatter stays.
     const size_t dn = (cg_dense_floats(sel->L) + cg_sten_floats(p.N, p.n_ubl)) * sizeof(float);
-    p.dense = o.solver == GC_LINCAL_CG && ctx->tune[GC_TUNE_CAL_OP] == 0 && !p.stencil && sel->L <= 64 &&
+    p.dense = o.solver == GC_LINCAL_CG && ctx->tune[GC_TUNE_CAL_OP] == 0 && !p.stencil && dense_tasks(sel->L) <= kCgDnThreads &&
                       16.0 * sel->P >= (double)p.N * p.N && dn <= kCgDnSmem
                   ? 1
                   : 0;
@@ -2430,7 +2437,7 @@ static gc_status fill_params(gc_ctx *ctx, gc_sel *sel, int C, const void *vreduc
     const bool fp64_ne = o.solver == GC_LINCAL && o.precision == GC_FP64;
     p.tol = o.tol > 0.0 ? o.tol : (fp64_ne ? 1e-10 : 1e-6);
     p.max_iter = o.max_iter > 0 ? o.max_iter : (o.solver == GC_OMNICAL ? 20000 : 50);
-    p.mu_rel = fp64_ne ? 1e-12 : 1e-7;
+    p.mu_rel = 1e-7;
     p.red32 = o.solver == GC_LINCAL_CG && o.fp32_reductions ? 1 : 0;
     p.work = nullptr;
     p.counter = nullptr;

@@ -737,15 +737,18 @@ int stage_mode(const void *volt, int L, bool tiled, size_t &smem) {
 using AccKernel = void (*)(const CUtensorMap, const Params);
 template <class K>
 AccKernel acc_kernel(int mode) {
-    return mode == kStageTiled ? fftcorr_accumulate<K, kStageTiled>
-                               : (mode == kStageBulk ? fftcorr_accumulate<K, kStageBulk> : fftcorr_accumulate<K, kStagePlain>);
+    if constexpr (K::M >= 64)   // (stage_mode)
+        if (mode == kStageBulk) return fftcorr_accumulate<K, kStageBulk>;
+    return mode == kStageTiled ? fftcorr_accumulate<K, kStageTiled> : fftcorr_accumulate<K, kStagePlain>;
 }
 
 // CTAs to launch for `items` equal items: k per SM, 1 <= k <= occ, for the
 // least time, k resident CTAs taking about k^a times as long for one item each
 // and the last wave as many as it has -- so a full last wave of fewer can beat
 // a nearly empty one.  Measured: a = 0.75 (two against one 1.55 to 1.67, three
-// against two 1.41), 0.35 for binary16 at M = 64 from bulk copies (1.13).
+// against two 1.41), 0.35 for binary16 at M = 64 from bulk copies (three against
+// two 1.13).  Its tiled form, two CTAs at most, has the same 0.35, not measured by
+// itself: it then launches two wherever that saves anything.
 int launch_ctas(long items, int occ, int sms, double a) {
     int best = 1;
     double least = 0.0;

@@ -247,6 +247,8 @@ __global__ void __launch_bounds__(kPThreads) xeng_pairs(const __grid_constant__ 
     }
 }
 
+// Entries per thread.  22 is the most whose offsets and sums fit 128 registers (the
+// limit at 512 threads): 23 spill in every format.
 constexpr int kKp[] = {22, 16, 12, 8, 4};
 
 template <int VF>
