@@ -2171,8 +2171,8 @@ lincal_cg_kernel(const CalParams p, double cg_tol, int cg_max, int smem_floats) 
     }
 }
 
-// The lag-plane operator (p.dense set): one CTA per SM, everything that the
-// operator reads in shared memory.
+// The lag-plane operator (p.dense set): everything that it reads in shared memory,
+// one CTA of kCgDnThreads per SM or several of fewer threads.
 __global__ void __launch_bounds__(kCgDnThreads, 1)
 lincal_cg_dense(const CalParams p, double cg_tol, int cg_max, int smem_floats, int coarse_smem) {
     __shared__ double red[32 * 14];
@@ -2509,7 +2509,15 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
         kfn = (const void *)omnical_kernel;
     }
     per_cta = (per_cta + 255) & ~size_t(255);
-    const int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? kCgStThreads : (p.dense ? kCgDnThreads : kCgThreads)) : kCThreads;
+    int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? kCgStThreads : (p.dense ? kCgDnThreads : kCgThreads)) : kCThreads;
+    // Lag planes for more channels than SMs: two CTAs of half the threads where
+    // they fit an SM (the scatter's two would otherwise be faster: 600 channels of
+    // the low-cadence 8x8 array, scatter 2.57 ms, one CTA 2.70, two 1.34; 16x16 22.5,
+    // 7.46 and 5.02).
+    if (p.dense && C > ctx->sm_count && dense_tasks(p.L) <= kCgDnThreads / 2) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, kCgDnThreads / 2, cg_smem);
+        if (e == cudaSuccess && occ >= 2) nthr = kCgDnThreads / 2;
+    }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, nthr, cg_smem);
     if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(calibration)");
     if (ctx->tune[GC_TUNE_CAL_CTAS] > 0) occ = std::min(occ, ctx->tune[GC_TUNE_CAL_CTAS]);
@@ -2528,7 +2536,7 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     if (o.solver == GC_LINCAL_CG) {
         const int sf = (int)(cg_smem / sizeof(float));
         if (p.stencil) lincal_cg_kernel<false, true><<<grid, kCgStThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
-        else if (p.dense) lincal_cg_dense<<<grid, kCgDnThreads, cg_smem, s>>>(p, 1e-4, 500, sf, dense_coarse);
+        else if (p.dense) lincal_cg_dense<<<grid, nthr, cg_smem, s>>>(p, 1e-4, 500, sf, dense_coarse);
         else if (!pipe) lincal_cg_kernel<false, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
         else lincal_cg_kernel<true, false><<<grid, kCgThreads, cg_smem, s>>>(p, 1e-4, 500, sf);
     } else {
