@@ -306,6 +306,17 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
         };
         if (kMode == kStageBulk && tid == 0) bulk_issue(t0);
         __syncthreads();
+        // On a grid short of the configuration the last item's parked sums (below)
+        // lie over rows that the column pass reads as zero: all threads clear them, as
+        // group 0 has read them by now and every staging form has a barrier ahead of
+        // the row pass.  (500 channels of 4x4 antennas, 1024 samples: 187 us; 196 with
+        // group 0 clearing what it reads.)
+        if constexpr (K::G > 1) {
+            static_assert(K::QG == 1, "one intermediate");
+            if (L < K::LMAX && item != (int)blockIdx.x)
+                for (int i = tid; i < (K::G - 1) * K::F2 * K::NCOL / 4; i += K::NTHREADS)
+                    reinterpret_cast<float4 *>(inter)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 
         float acc[K::F2];
 #pragma unroll
@@ -467,9 +478,7 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
 
         // chunk spectrum P[k_y][k_x]: the groups hold the same bins for
         // different samples; groups 1.. park theirs in the (now idle)
-        // intermediate buffer and group 0 adds them up and stores.  On a grid
-        // short of the configuration the parked sums lie over rows that the
-        // next item's column pass reads as zero: their reader clears them
+        // intermediate buffer and group 0 adds them up and stores
         if constexpr (K::G > 1) {
             float *park = reinterpret_cast<float *>(inter);
             if (g > 0) {
@@ -480,11 +489,7 @@ fftcorr_accumulate(const __grid_constant__ CUtensorMap tmap, const Params p) {
             if (g == 0) {
 #pragma unroll
                 for (int i = 0; i < K::F2; ++i)
-                    for (int gg = 1; gg < K::G; ++gg) {
-                        float &q = park[((gg - 1) * K::F2 + i) * K::NCOL + col];
-                        acc[i] += q;
-                        if (L < K::LMAX) q = 0.f;
-                    }
+                    for (int gg = 1; gg < K::G; ++gg) acc[i] += park[((gg - 1) * K::F2 + i) * K::NCOL + col];
             }
         }
         if (g == 0) {
