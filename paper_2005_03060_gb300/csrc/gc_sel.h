@@ -18,7 +18,7 @@ struct gc_sel {
     std::vector<int32_t> win_t0, win_t1;              // [n_ubl]
     // neighbour table [2][n_ubl][N]: pair index with antenna i as i_p (0) or
     // as j_p (1), -1 if none; empty when it would exceed 16 M entries, and for
-    // full grids of more than 64 types
+    // full grids of more than 160 types
     std::vector<int32_t> nbr;
     // X-engine work groups (types sharing a window, <= GC_XENG_NTY each)
     int n_groups = 0, n_windows = 0;

@@ -104,11 +104,12 @@ void fill_pairs(gc_sel *s) {
     }
     s->P = (int)s->pair_i.size();
     // (on a full grid only omnical reads it, and for many types arithmetic is
-    // faster: 12x12 antennas, 264 types, 10.6 against 17.9 ms; 6x6, 60 types,
-    // 4.1 against 3.4 ms)
+    // faster.  Table against arithmetic, 64 channels: 8x8 antennas, 112 types, 4.2
+    // and 4.7 ms; 9x9, 144 types, 5.5 and 6.1; 10x10, 180 types, 7.5 and 6.9; 12x12,
+    // 264 types, 16.5 and 9.5)
     const size_t N = (size_t)L * L;
     s->nbr.clear();
-    if ((s->masked || s->n_ubl <= 64) && 2 * (size_t)s->n_ubl * N <= (16u << 20)) {
+    if ((s->masked || s->n_ubl <= 160) && 2 * (size_t)s->n_ubl * N <= (16u << 20)) {
         s->nbr.assign(2 * (size_t)s->n_ubl * N, -1);
         for (int q = 0; q < s->P; ++q) {
             const int k = s->pair_type[q];
