@@ -1039,11 +1039,12 @@ __device__ double dense_resid_pass(const CalParams &p, int c, const CgWork &w, b
     }
     __syncthreads();
     float chi = 0.f;
+    const float so = unit_scale().o;
     const float2 *vf = reinterpret_cast<const float2 *>(p.vred) + (size_t)c * p.P;
     const int2 *vi = reinterpret_cast<const int2 *>(p.vred) + (size_t)c * p.P;
     float *hb = reinterpret_cast<float *>(w.yb);
     for (int k = wp; k < K; k += nw) {
-        const float inv = unit_scale().o * (1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)));
+        const float inv = so * (1.0f / (float)(__ldg(p.win_t1 + k) - __ldg(p.win_t0 + k)));
         const float Vx = xv[2 * k], Vy = xv[2 * k + 1];
         float tx = 0.f, ty = 0.f, td = 0.f;
         const int q1 = __ldg(p.type_ptr + k + 1);
@@ -2510,13 +2511,15 @@ extern "C" gc_status gc_calibrate(gc_ctx *ctx, const void *vreduced, int vfmt, c
     }
     per_cta = (per_cta + 255) & ~size_t(255);
     int nthr = o.solver == GC_LINCAL_CG ? (p.stencil ? kCgStThreads : (p.dense ? kCgDnThreads : kCgThreads)) : kCThreads;
-    // Lag planes for more channels than SMs: two CTAs of half the threads where
-    // they fit an SM (the scatter's two would otherwise be faster: 600 channels of
-    // the low-cadence 8x8 array, scatter 2.57 ms, one CTA 2.70, two 1.34; 16x16 22.5,
-    // 7.46 and 5.02).
-    if (p.dense && C > ctx->sm_count && dense_tasks(p.L) <= kCgDnThreads / 2) {
+    // Lag planes by half the threads: for more channels than SMs where two such CTAs
+    // fit an SM (the scatter's two would otherwise be faster: 600 channels of the
+    // low-cadence 8x8 array, scatter 2.57 ms, one CTA 2.70, two 1.34; 16x16 22.5, 7.46
+    // and 5.02), and on grids of up to 10x10, whose few tasks the barriers of 512
+    // threads outweigh (64 channels: 4x4 0.58 ms by 512 threads, 0.47 by 256, scatter
+    // 0.65; 10x10 0.87 and 0.80; 12x12 1.06 and 1.09).
+    if (p.dense && dense_tasks(p.L) <= kCgDnThreads / 2) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, kCgDnThreads / 2, cg_smem);
-        if (e == cudaSuccess && occ >= 2) nthr = kCgDnThreads / 2;
+        if (p.L <= 10 || (C > ctx->sm_count && e == cudaSuccess && occ >= 2)) nthr = kCgDnThreads / 2;
     }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, nthr, cg_smem);
     if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(calibration)");
