@@ -68,7 +68,8 @@ struct gc_xeng_pairs_shape {
 // elements per staged grid row: two spare ones where rows of a multiple of 8
 // would put a column of antennas on one bank
 inline int gc_xeng_pairs_pitch(int L) { return L % 8 == 0 ? L + 2 : L; }
-bool gc_xeng_pairs_eligible(const gc_sel *sel, int vfmt);
-gc_status gc_xeng_pairs_plan(gc_ctx *ctx, const gc_sel *sel, int vfmt, int C, bool autos, gc_xeng_pairs_shape *sh);
+bool gc_xeng_pairs_eligible(const gc_ctx *ctx, const gc_sel *sel, int vfmt, int C);
+bool gc_xeng_pairs_bulk(const gc_sel *sel, int vfmt, const void *volt);
+gc_status gc_xeng_pairs_plan(gc_ctx *ctx, const gc_sel *sel, int vfmt, int C, bool autos, bool bulk, gc_xeng_pairs_shape *sh);
 gc_status gc_xeng_pairs_launch(gc_ctx *ctx, const void *volt, int vfmt, int C, int T, const gc_sel *sel,
                                const gc_xeng_pairs_shape &sh, void *out, void *apart, cudaStream_t s);

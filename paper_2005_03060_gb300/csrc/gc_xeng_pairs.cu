@@ -285,29 +285,35 @@ size_t pairs_smem(int vfmt, int L, size_t &stride) {
 
 }  // namespace
 
-// Several windows, and two samples of the grid fit the stages.
-bool gc_xeng_pairs_eligible(const gc_sel *sel, int vfmt) {
+// Several windows, and two samples of the grid fit the stages.  Not: binary16 on
+// rows of a multiple of 32 (staged as they lie, columns share banks) where few
+// channels have long windows -- 32x32 antennas, 4096 samples, one channel 111 us,
+// 91 in the antenna form; two 181 and 168; four 316 and 322.
+bool gc_xeng_pairs_eligible(const gc_ctx *ctx, const gc_sel *sel, int vfmt, int C) {
     size_t stride;
     if (sel->masked && sel->nbr.empty()) return false;   // refused without the pair table
-    return !sel->wp_entry.empty() && pairs_smem(vfmt, sel->L, stride) <= 200u * 1024u;
+    if (sel->wp_entry.empty() || pairs_smem(vfmt, sel->L, stride) > 200u * 1024u) return false;
+    return !(vfmt == GC_C32H && sel->L % 32 == 0 && (long)C * sel->n_windows < ctx->sm_count && sel->t_int >= 64);
 }
 
-gc_status gc_xeng_pairs_plan(gc_ctx *ctx, const gc_sel *sel, int vfmt, int C, bool autos, gc_xeng_pairs_shape *sh) {
-    const int N = sel->L * sel->L;
-    int most = 0, max_win = 0;
-    for (int w = 0; w < sel->n_windows; ++w) {
-        most = std::max(most, sel->wp_off[w + 1] - sel->wp_off[w] - (autos ? 0 : N));
-        max_win = std::max(max_win, sel->wp_t1[w] - sel->wp_t0[w]);
-    }
-    // entries per thread: the fewest idle slots among the shapes of at least
-    // 128 threads (more entries a thread hide the read latency better and
-    // are listed first); a window past 512 threads is split into blocks
+// Staged by copy engines: whole 16-byte units a sample.
+bool gc_xeng_pairs_bulk(const gc_sel *sel, int vfmt, const void *volt) {
+    return gc_aligned(volt, 16) && ((size_t)sel->L * sel->L * elem_size(vfmt)) % 16 == 0;
+}
+
+namespace {
+
+// Entries per thread, threads and blocks of a window of `most` entries in at
+// least `least` blocks: the fewest idle slots among the shapes of at least 128
+// threads (more entries a thread hide the read latency better and are listed
+// first); a window past 512 threads is split into blocks.
+void pairs_blocks(int most, int least, gc_xeng_pairs_shape *sh) {
+    const int per1 = (most + least - 1) / least;
     sh->kp = 4;
-    sh->n_blk = 1;
-    sh->nthr = std::min(kPThreads, std::max(32, ((most + 3) / 4 + 31) / 32 * 32));
+    sh->nthr = std::min(kPThreads, std::max(32, ((per1 + 3) / 4 + 31) / 32 * 32));
     long best = -1;
     for (int kp : kKp) {
-        const int nb = (most + kPThreads * kp - 1) / (kPThreads * kp);
+        const int nb = std::max(least, (most + kPThreads * kp - 1) / (kPThreads * kp));
         const int per = (most + nb - 1) / nb;
         const int nthr = ((per + kp - 1) / kp + 31) / 32 * 32;
         if (nthr < 128 && kp > 4) continue;
@@ -315,39 +321,105 @@ gc_status gc_xeng_pairs_plan(gc_ctx *ctx, const gc_sel *sel, int vfmt, int C, bo
         if (best < 0 || slots < best) {
             best = slots;
             sh->kp = kp;
-            sh->n_blk = nb;
             sh->nthr = nthr;
         }
     }
     sh->per_blk = sh->nthr * sh->kp;
     sh->n_blk = (most + sh->per_blk - 1) / sh->per_blk;
+}
+
+// Cycles that a reduction whose items all fit the chip takes in ts time slices: an
+// item's start (first copies, then entry lists and scattered stores), its samples,
+// each with the products' latency, the shared-memory reads of the SM's `live` CTAs
+// at 128 B a cycle (16, 8 or 6 bytes an entry) and what the threads themselves
+// stage or expand; then the partial sums of the slices, and the autocorrelations
+// of all windows and slices.  The constants are from runs of few channels, 3x3 to 32x32 antennas.
+double pairs_cycles(const gc_sel *sel, int vfmt, int C, int sms, int max_win, bool bulk, const gc_xeng_pairs_shape &sh,
+                    int ts) {
+    const int N = sel->L * sel->L;
+    const double bytes = vfmt == GC_C64 ? 16.0 : (vfmt == GC_C32H ? 8.0 : 6.0);
+    const double live = (double)(((long)C * sel->n_windows * sh.n_blk * ts + sms - 1) / sms);
+    double sample = 150.0 + live * sh.per_blk * bytes / 128.0;
+    if (vfmt == GC_I4C) sample += 100.0 + 8.0 * N / sh.nthr;
+    if (!bulk) sample += 20.0 * N / sh.nthr;
+    double t = 5000.0 + 2.5 * live * sh.per_blk + (double)((max_win + ts - 1) / ts) * sample;
+    if (ts > 1) t += 100.0 * ts + (double)ts * C * sel->P * 16.0 / 3500.0;
+    return t + 40.0 * ts * sel->n_windows;
+}
+
+}  // namespace
+
+gc_status gc_xeng_pairs_plan(gc_ctx *ctx, const gc_sel *sel, int vfmt, int C, bool autos, bool bulk, gc_xeng_pairs_shape *sh) {
+    int most = 0, max_win = 0;   // (window's pairs and autocorrelations)
+    for (int w = 0; w < sel->n_windows; ++w) {
+        most = std::max(most, sel->wp_off[w + 1] - sel->wp_off[w]);
+        max_win = std::max(max_win, sel->wp_t1[w] - sel->wp_t0[w]);
+    }
+    pairs_blocks(most, 1, sh);
     sh->smem = pairs_smem(vfmt, sel->L, sh->stage_stride);
-    sh->ns = stage_samples(vfmt, (size_t)N * elem_size(vfmt));
-    sh->kern = vfmt == GC_C64 ? pick_pairs<GC_C64>(sh->kp)
-                              : (vfmt == GC_C32H ? pick_pairs<GC_C32H>(sh->kp) : pick_pairs<GC_I4C>(sh->kp));
-    cudaError_t e = cudaFuncSetAttribute(sh->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(xeng_pairs)");
+    sh->ns = stage_samples(vfmt, (size_t)sel->L * sel->L * elem_size(vfmt));
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sh->kern, sh->nthr, sh->smem);
-    if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(xeng_pairs)");
-    const int slots = occ * ctx->sm_count;
+    auto resident = [&]() {
+        sh->kern = vfmt == GC_C64 ? pick_pairs<GC_C64>(sh->kp)
+                                  : (vfmt == GC_C32H ? pick_pairs<GC_C32H>(sh->kp) : pick_pairs<GC_I4C>(sh->kp));
+        cudaError_t e = cudaFuncSetAttribute(sh->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        if (e != cudaSuccess) return gc_cuda_fail(ctx, e, "cudaFuncSetAttribute(xeng_pairs)");
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sh->kern, sh->nthr, sh->smem);
+        if (e != cudaSuccess || occ < 1) return gc_cuda_fail(ctx, e, "occupancy(xeng_pairs)");
+        return GC_OK;
+    };
+    gc_status st = resident();
+    if (st != GC_OK) return st;
     // split long windows in time so that the items fill whole waves of the
     // resident CTAs (slices of at least 64 samples)
-    const long base = (long)C * sel->n_windows * sh->n_blk;
+    const int slots = occ * ctx->sm_count;
+    const long base = (long)C * sel->n_windows;
     sh->n_tsplit = 1;
     double top = -1.0;
-    for (int ts = 1; ts <= 16; ++ts) {
-        if (ts > 1 && max_win / ts < 64) break;
-        const long items = base * ts, waves = (items + slots - 1) / slots;
+    for (int ts = 1; ts <= 16 && (ts == 1 || max_win / ts >= 64); ++ts) {
+        const long items = base * sh->n_blk * ts, waves = (items + slots - 1) / slots;
         const double eff = (double)items / ((double)waves * slots) - 0.01 * ts;   // prefer fewer slices
         if (eff > top) {
             top = eff;
             sh->n_tsplit = ts;
         }
     }
+    // Where that leaves SMs idle (few channels: there the 0.01 outweighs the fill):
+    // slices down to 16 samples, and blocks of a window on several SMs, each of
+    // which stages the window's samples again, by the cycles they are reckoned to
+    // take and if these are fewer by a quarter.  One channel, without / so / in the
+    // antenna form: 8x8 antennas, 8192 complex64 samples 133 / 29 / 33 us; 6x6, 8192
+    // samples of 4+4 bits 289 / 25 / 25; 32x32, 4096 complex64 samples 93 / 64 / 85.
+    if (base * sh->n_blk * sh->n_tsplit < ctx->sm_count) {
+        gc_xeng_pairs_shape best = *sh;
+        double least = 0.75 * pairs_cycles(sel, vfmt, C, ctx->sm_count, max_win, bulk, *sh, sh->n_tsplit);
+        for (int nb = sh->n_blk; nb <= 16; nb *= 2) {
+            gc_xeng_pairs_shape more = *sh;
+            if (nb > sh->n_blk) pairs_blocks(most, nb, &more);
+            if (nb > sh->n_blk && more.nthr < 128) break;
+            const long fit = nb > sh->n_blk ? ctx->sm_count : slots;
+            for (int ts = 1; ts <= 64 && (ts == 1 || max_win / ts >= 16) && base * more.n_blk * ts <= fit; ++ts) {
+                const double t = pairs_cycles(sel, vfmt, C, ctx->sm_count, max_win, bulk, more, ts);
+                if (t < least) {
+                    least = t;
+                    best = more;
+                    best.n_tsplit = ts;
+                }
+            }
+        }
+        *sh = best;
+        st = resident();
+        if (st != GC_OK) return st;
+    }
+    // without autocorrelations the same slices (the same sums, bit for bit) in smaller blocks
+    if (!autos) {
+        pairs_blocks(most - sel->L * sel->L, sh->n_blk, sh);
+        st = resident();
+        if (st != GC_OK) return st;
+    }
     if (ctx->tune[GC_TUNE_XENG_TSPLIT] > 0) sh->n_tsplit = std::min(ctx->tune[GC_TUNE_XENG_TSPLIT], 64);
-    sh->n_items = base * sh->n_tsplit;
-    sh->grid = (int)std::min<long>(sh->n_items, slots);
+    sh->n_items = (long)C * sel->n_windows * sh->n_blk * sh->n_tsplit;
+    sh->grid = (int)std::min<long>(sh->n_items, (long)occ * ctx->sm_count);
     return GC_OK;
 }
 
@@ -377,7 +449,7 @@ gc_status gc_xeng_pairs_launch(gc_ctx *ctx, const void *volt, int vfmt, int C, i
     p.apart = apart;
     p.status = ctx->status_dev;
     p.stage_stride = sh.stage_stride;
-    p.use_tma = gc_aligned(volt, 16) && ((size_t)p.N * elem_size(vfmt)) % 16 == 0 ? 1 : 0;
+    p.use_tma = gc_xeng_pairs_bulk(sel, vfmt, volt) ? 1 : 0;
     p.pitch = pairs_pitch(vfmt, p.L);
     CUtensorMap tmap;
     memset(&tmap, 0, sizeof tmap);

@@ -428,9 +428,9 @@ extern "C" gc_status gc_reduce(gc_ctx *ctx, const void *volt, int vfmt, int L, i
     }
     // several windows (low-cadence): the pair-list form, which writes
     // V^reduced itself when the windows are not split in time
-    if (gc_xeng_pairs_eligible(sel, vfmt)) {
+    if (gc_xeng_pairs_eligible(ctx, sel, vfmt, C)) {
         gc_xeng_pairs_shape sh;
-        st = gc_xeng_pairs_plan(ctx, sel, vfmt, C, autos != nullptr, &sh);
+        st = gc_xeng_pairs_plan(ctx, sel, vfmt, C, autos != nullptr, gc_xeng_pairs_bulk(sel, vfmt, volt), &sh);
         if (st != GC_OK) return st;
         const bool direct = sh.n_tsplit == 1;
         const size_t part_bytes = direct ? 0 : ((size_t)sh.n_tsplit * C * sel->P * sizeof(float2) + 255) / 256 * 256;
