@@ -65,9 +65,10 @@ def flops_per_antenna_sample(L: int, M: int) -> float:
 
 
 def lincal_flops_per_iter(P: int) -> float:
-    """FP64 flops of one Gauss-Newton iteration of the direct solver: the
-    gradient and chi^2, 24 FP64 multiply-adds a pair (the step's matrix is
-    factorised in FP32)."""
+    """FP64 flops that a Gauss-Newton iteration of the direct solver cannot do
+    without: the gradient and chi^2, 24 FP64 multiply-adds a pair (the step's
+    matrix is factorised in FP32; refinement passes, the first and the last
+    evaluation and halved steps come on top)."""
     return 48.0 * P
 
 
@@ -891,6 +892,7 @@ def run_ours(args, rank, world, local_rank):
         v64 = variants["lincal_fp64"]
         flops = v64["channels"] * v64["mean_iters"] * lincal_flops_per_iter(w.sel.P)
         v64["fp64_frac"] = flops / (v64["ms"] * 1e-3) / 1e12 / probes["fp64"]
+        v64["fp64_frac_of"] = "one gradient and chi^2 per iteration, the least FP64 work; not what bounds the solver"
     dom = max(kern.items(), key=lambda kv: kv[1][0])[0]
     roofline = dict(rl.get(dom, {"bound": "unknown"}))
     roofline["kernel"] = dom

@@ -297,7 +297,8 @@ GC_API gc_status gc_quantize(gc_ctx *ctx, const float *volt, int C, int T, int N
  *              occupied lattices.
  * Start point (unless warm_start): spanning-tree phases over the (1,0) and
  * (0,1) types, unit amplitudes, group-mean model visibilities.  Warm start
- * reads gains and vmodel as given.
+ * reads gains and vmodel as given (GC_LINCAL_CG: elements of exactly zero
+ * first take least-squares values from the others).
  * Output convention for the degeneracies: mean ln|g| = 0, arg g_0 = 0,
  * arg V_(1,0) = arg V_(0,1) = 0.
  *
